@@ -2066,10 +2066,21 @@ __global__ void __launch_bounds__(32) k_search_paper(const Dev<W> a)
 // frontier offsets (exclusive scan of the record counts) and opens the
 // step's first search pass, which reads the frontiers in place.
 // ---------------------------------------------------------------------
-template <int W> struct SplitShared {
-    static constexpr int CAP = (W <= 4) ? 512 : 384;  // records per shared level buffer
+//
+// A level is a few hundred cycles of latency, so what counts is how many
+// barriers and dependent steps it has: a thread expands one record, children
+// stay in registers (never indexed dynamically), their places come from
+// ballots within the warp and one barrier for the warps' totals, and the
+// counts that only the end needs are reduced there. (Before, with an indexed
+// array of children and two block scans of three barriers per level, it was
+// 10 to 136 us of every step: half of the time of 5000 8-puzzles in one call,
+// 2065 -> 1710 us; one-board calls with 6-6-3 pattern databases 3.00 -> 2.71 ms,
+// one 24-puzzle 445 -> 420 us.)
+// SMALLB: blocks of 128 threads, for calls whose frontiers are short.
+template <int W, bool SMALLB = false> struct SplitShared {
+    static constexpr int CAP = SMALLB ? 128 : (W <= 4) ? 512 : 384;  // records per shared level buffer
 };
-static constexpr int SPLIT_THREADS = 512;
+static constexpr int SPLIT_THREADS = 512, SPLIT_THREADS_SMALL = 128;
 
 template <int W>
 __device__ __forceinline__ bool last_block_done(unsigned *counter, int *s_last)
@@ -2088,16 +2099,17 @@ __device__ __forceinline__ bool last_block_done(unsigned *counter, int *s_last)
     return false;
 }
 
-template <int W, bool PDB = false>
-__global__ void __launch_bounds__(SPLIT_THREADS) k_split(const Dev<W> a)
+template <int W, bool PDB = false, bool SMALLB = false>
+__global__ void __launch_bounds__(SMALLB ? SPLIT_THREADS_SMALL : SPLIT_THREADS) k_split(const Dev<W> a)
 {
     typedef typename Geo<W>::B B;
     constexpr int BITS = Geo<W>::BITS;
-    constexpr int SCAP = SplitShared<W>::CAP;
+    constexpr int SCAP = SplitShared<W, SMALLB>::CAP;
+    constexpr int NT = SMALLB ? SPLIT_THREADS_SMALL : SPLIT_THREADS, NW = NT / 32;
     __shared__ __align__(16) unsigned char lut[SharedLut<W>::BYTES];
     __shared__ Rec<W> lvl[2][SCAP];
-    __shared__ int warp_sums[32];
-    __shared__ int s_fmin, s_last, s_carry;
+    __shared__ int warp_sums[32], level_sums[2][NW];
+    __shared__ int s_fmin, s_last;
     __shared__ unsigned long long s_internal;
     __shared__ unsigned s_low[FUSE_MAX];  // expanded nodes with slack 2m, m < J (fused steps)
 
@@ -2158,6 +2170,10 @@ __global__ void __launch_bounds__(SPLIT_THREADS) k_split(const Dev<W> a)
         int cnt = 1, depth = 0;
         int expandable = (st.root == GOAL) ? 0 : 1;
         Rec<W> *cur = lvl[0];
+        const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+        const unsigned lt = (1u << lane) - 1u;
+        int fmin = INT_MAX, turn = 0;
+        unsigned internal = 0;  // records this thread expanded
         for (;;) {
             // the root is always expanded here (unless it is the goal): every
             // record the search kernel receives then has a parent move, so a
@@ -2171,32 +2187,26 @@ __global__ void __launch_bounds__(SPLIT_THREADS) k_split(const Dev<W> a)
             else
                 nxt = (cur == A) ? Bg : A;
             int outbase = 0, nonleaf = 0;
-            int fmin = INT_MAX;
-            unsigned long long internal = 0;
-            for (int base = 0; base < cnt; base += blockDim.x) {
+            for (int base = 0; base < cnt; base += NT) {
                 const int j = base + threadIdx.x;
-                Rec<W> r;
-                r.meta = M_LEAF;
                 const bool v = j < cnt;
+                Rec<W> r;
+                r.meta = 0;
                 if (v)
                     r = cur[j];
                 const bool leaf = v && (r.meta & M_LEAF);
-                const bool exp = v && !leaf;
-                Rec<W> c[4];
-                int nc = 0, nl = 0;
-                if (leaf) {
-                    c[0] = r;
-                    nc = 1;
-                } else if (exp) {
+                const int p = (int)m_blank(r.meta);
+                const int s = m_slack(r.meta);
+                // kept children, the goal among them, and the moves away from
+                // the goal cell, by move; the children's boards
+                unsigned kept = 0, goals = 0, away4 = 0;
+                B cb[4];
+                if (v && !leaf) {
                     internal += 1;
-                    const int p = (int)m_blank(r.meta);
                     const int last = (int)m_last(r.meta);
-                    const int s = m_slack(r.meta);
                     if (s < 2 * J)
                         atomicAdd(&s_low[s >> 1], 1u);
-                    const uint32_t d = m_hi(r.meta);
                     const LutRow<W> e = SharedLut<W>::row(lut, p);
-                    unsigned away4 = 0;
                     if constexpr (PDB) {
                         // the four moves' table reads together (see pdb_away4)
                         const uint64_t inv = pdb_inverse<W>(r.b, *pi);
@@ -2213,55 +2223,71 @@ __global__ void __launch_bounds__(SPLIT_THREADS) k_split(const Dev<W> a)
                     }
 #pragma unroll
                     for (int m = 0; m < 4; ++m) {
-                        if (!e.legal(m) || last == 3 - m)
-                            continue;
-                        const int np = p + move_off<W>(m);
-                        const unsigned t = tile_at<W>(r.b, np);
-                        bool away;
-                        if constexpr (PDB)
-                            away = (away4 >> m) & 1u;
-                        else
-                            away = e.away(m, t);
-                        const int s2 = away ? s - 2 : s;
-                        if (s2 < 0) {
-                            fmin = min(fmin, -s2);
-                            continue;
+                        cb[m] = 0;
+                        if (e.legal(m) && last != 3 - m) {
+                            const int np = p + move_off<W>(m);
+                            const unsigned t = tile_at<W>(r.b, np);
+                            if constexpr (!PDB)
+                                away4 |= (e.away(m, t) ? 1u : 0u) << m;
+                            const B x = (B)t;
+                            cb[m] = r.b + (x << (BITS * p)) - (x << (BITS * np));
+                            if (((away4 >> m) & 1u) && s < 2) {
+                                fmin = min(fmin, 2 - s);
+                            } else {
+                                kept |= 1u << m;
+                                goals |= (cb[m] == GOAL ? 1u : 0u) << m;
+                            }
                         }
-                        const B x = (B)t;
+                    }
+                }
+                // places: the prefix of the counts (0..4) over the block
+                const unsigned nc = leaf ? 1u : (unsigned)__popc(kept);
+                const unsigned b0 = __ballot_sync(FULL, nc & 1u), b1 = __ballot_sync(FULL, nc & 2u),
+                               b2 = __ballot_sync(FULL, nc & 4u);
+                const unsigned open = __reduce_add_sync(FULL, (unsigned)__popc(kept & ~goals));
+                int *sums = level_sums[turn & 1];
+                ++turn;
+                if (lane == 0)
+                    sums[wid] = (__popc(b0) + 2 * __popc(b1) + 4 * __popc(b2)) | (int)(open << 16);
+                __syncthreads();
+                const unsigned x = lane < NW ? (unsigned)sums[lane] : 0u;
+                const unsigned total = __reduce_add_sync(FULL, x);
+                const unsigned before = __reduce_add_sync(FULL, lane < wid ? x & 0xffffu : 0u);
+                Rec<W> *at = nxt + outbase + before + __popc(b0 & lt) + 2 * __popc(b1 & lt) + 4 * __popc(b2 & lt);
+                if (leaf)
+                    *at = r;
+                const uint32_t d = m_hi(r.meta);
+#pragma unroll
+                for (int m = 0; m < 4; ++m)
+                    if ((kept >> m) & 1u) {
                         Rec<W> ch;
-                        ch.b = r.b + (x << (BITS * p)) - (x << (BITS * np));
-                        ch.meta = (uint32_t)np | ((uint32_t)m << 5) | ((uint32_t)s2 << 8) | ((d + 1u) << 16);
-                        if (ch.b == GOAL)
-                            ch.meta |= M_LEAF;
-                        else
-                            ++nl;
+                        ch.b = cb[m];
+                        ch.meta = (uint32_t)(p + move_off<W>(m)) | ((uint32_t)m << 5) |
+                                  ((uint32_t)(((away4 >> m) & 1u) ? s - 2 : s) << 8) | ((d + 1u) << 16) |
+                                  (((goals >> m) & 1u) ? M_LEAF : 0u);
                         ch.inst = inst;
                         ch.origin = 0;
                         ch.pm = r.pm | ((uint32_t)m << (2 * d));
-                        c[nc++] = ch;
+                        at[__popc(kept & ((1u << m) - 1u))] = ch;
                     }
-                }
-                // one scan for both counts: records (low half), expandable records (high half)
-                int total;
-                const int pos = block_exclusive_scan(nc | (nl << 16), warp_sums, &total);
-                for (int q = 0; q < nc; ++q)
-                    nxt[outbase + (pos & 0xffff) + q] = c[q];
-                outbase += total & 0xffff;
-                nonleaf += total >> 16;
+                outbase += (int)(total & 0xffffu);
+                nonleaf += (int)(total >> 16);
             }
-            fmin = warp_min_int(fmin);
-            if ((threadIdx.x & 31) == 0)
-                atomicMin(&s_fmin, fmin);
-            for (int d2 = 16; d2; d2 >>= 1)
-                internal += __shfl_xor_sync(FULL, internal, d2);
-            if ((threadIdx.x & 31) == 0)
-                atomicAdd(&s_internal, internal);
             __syncthreads();
             cur = nxt;
             cnt = outbase;
             expandable = nonleaf;
             ++depth;
         }
+        fmin = warp_min_int(fmin);
+        internal = __reduce_add_sync(FULL, internal);
+        if (lane == 0) {
+            if (fmin != INT_MAX)
+                atomicMin(&s_fmin, fmin);
+            if (internal)
+                atomicAdd(&s_internal, (unsigned long long)internal);
+        }
+        __syncthreads();
         if (cur != A) {
             for (int j = threadIdx.x; j < cnt; j += blockDim.x)
                 A[j] = cur[j];
@@ -2283,34 +2309,34 @@ __global__ void __launch_bounds__(SPLIT_THREADS) k_split(const Dev<W> a)
     }
     if (!last_block_done<W>((unsigned *)&ctrl->done_blocks, &s_last))
         return;
-    // last block: frontier offsets, then open the first pass of the step
-    if (threadIdx.x == 0)
-        s_carry = 0;
-    __syncthreads();
+    // last block: frontier offsets (each thread a run of consecutive problems),
+    // then open the first pass of the step
     const unsigned *act = ctrl->cur ? a.act1 : a.act0;
-    for (int base = 0; base < n_active; base += blockDim.x) {
-        const int j = base + threadIdx.x;
-        const int v = j < n_active ? __ldcg(&a.count[j]) : 0;
-        int total;
-        const int pos = block_exclusive_scan(v, warp_sums, &total);
-        if (j < n_active)
-            a.offset[j] = s_carry + pos;
-        if (j < n_active && a.slice && v > 0) {
+    const int per = (n_active + NT - 1) / NT;
+    const int k0 = min(n_active, (int)threadIdx.x * per), k1 = min(n_active, k0 + per);
+    int mine = 0, n_front;
+#pragma unroll 4
+    for (int j = k0; j < k1; ++j)
+        mine += __ldcg(&a.count[j]);
+    int off = block_exclusive_scan(mine, warp_sums, &n_front);
+#pragma unroll 4
+    for (int j = k0; j < k1; ++j) {
+        const int v = __ldcg(&a.count[j]);
+        a.offset[j] = off;
+        if (a.slice && v > 0) {
             // the frontier numbering of this iteration, kept while it runs
-            a.fbase[act[j]] = s_carry + pos;
+            a.fbase[act[j]] = off;
             a.fcount[act[j]] = v;
         }
-        __syncthreads();
-        if (threadIdx.x == 0)
-            s_carry += total;
-        __syncthreads();
+        off += v;
     }
+    __syncthreads();
     if (threadIdx.x == 0) {
         ctrl->done_blocks = 0;
         // the first pass reads the frontiers, then the carried open nodes
         const int carried = a.slice ? ctrl->n_carry : 0;
-        ctrl->n_front = s_carry;
-        ctrl->n_in = s_carry + carried;
+        ctrl->n_front = n_front;
+        ctrl->n_in = n_front + carried;
         ctrl->head = 0;
         ctrl->out_count = 0;
         ctrl->exited = 0;
@@ -2322,7 +2348,7 @@ __global__ void __launch_bounds__(SPLIT_THREADS) k_split(const Dev<W> a)
         ctrl->t_start = ~0ull;
         ctrl->t_end = 0;
         ctrl->done_warps = 0;
-        ctrl->records_total += (unsigned long long)s_carry;
+        ctrl->records_total += (unsigned long long)n_front;
         __threadfence();
         if (a.graph)
             cudaGraphSetConditional(a.h_pass, 1u);
