@@ -24,6 +24,7 @@
 // after every pass (it synchronises the stream); it is what times each
 // search launch with CUDA events.
 #include "bpida.h"
+#include "bpida_chain.cuh"
 #include "bpida_device.cuh"
 #include "bpida_pdb.h"
 #include "bpida_thread.h"
@@ -297,13 +298,36 @@ struct Geometry {
     int n_cap;
     int variant;
     bool fuse;
+    int chain;  // k_search_chain: its warps per block, else 0
 };
+
+// 15-puzzle calls of at least CHAIN_MIN_N boards search with k_search_chain.
+// It is the faster one wherever the search itself is the time (random
+// permutations: 64 boards 229.7 ms against 300.4 with k_search, 16 boards 42.0
+// against 51.9), and the slower one on short searches, whose time is how soon
+// a record spreads over a warp's lanes (40-move walks: 16 boards 1150 us
+// against 1050, 64 boards 1686 against 1546). The number of boards does not
+// tell the two apart; the line lies where a batch is more likely to hold a
+// hard board, and below it easy small calls keep the shorter time.
+constexpr int CHAIN_MIN_N = 64;
+// Its stack entries per lane: 20 where they fit (five 4-warp blocks per SM;
+// every block size that a caller can ask for leaves room for 13).
+int chain_entries(int wpb, size_t lim)
+{
+    int cap = 20;
+    while (cap > 12 && Chain::BYTES + wpb * ChainStack::bytes(cap) > lim)
+        --cap;
+    return cap;
+}
 
 // variant 0: warp per subtree group; 1: the paper's kernel; 6: block per
 // subtree group (the autotuner's other mode, widths 3 and 4)
 constexpr int VARIANT_BLOCK = 6;
-template <int W, int S, bool PDB> void (*search_kernel(int variant, bool fuse))(const Dev<W>)
+template <int W, int S, bool PDB> void (*search_kernel(int variant, bool fuse, int chain))(const Dev<W>)
 {
+    if constexpr (W == 4 && !PDB)
+        if (chain)
+            return chain > CHAIN_WARPS ? k_search_chain<64> : k_search_chain<>;
     if constexpr (PDB) {
         return fuse ? k_search<W, S, true, true> : k_search<W, S, false, true>;
     } else {
@@ -372,7 +396,7 @@ cudaError_t build_graph(Plan &pl, Dev<W> d, const Geometry &g, const char **wher
 
     cudaGraphNode_t n_search;
     *where = "search node";
-    if ((e = add_kernel(&n_search, P, nullptr, 0, search_kernel<W, S, PDB>(g.variant, g.fuse), dim3(g.grid), dim3(g.threads),
+    if ((e = add_kernel(&n_search, P, nullptr, 0, search_kernel<W, S, PDB>(g.variant, g.fuse, g.chain), dim3(g.grid), dim3(g.threads),
                         g.smem, d)) != cudaSuccess)
         return e;
     *where = "cudaGraphInstantiate";
@@ -402,28 +426,35 @@ bpida_status run(const Settings &cfg, const uint64_t *boards, int n, int *out_le
     g.fuse = fuse;
     const int wpb = cfg.variant == 1 ? 1 : cfg.wpb;  // the paper's kernel: block = warp
     g.threads = wpb * 32;
+    g.chain = (W == 4 && !PDB && cfg.variant == 0 && n >= CHAIN_MIN_N) ? wpb : 0;
+    const int form = (fuse ? 1 : 0) + (g.chain ? (wpb > CHAIN_WARPS ? 4 : 2) : 0);
     // search stack entries: 16 bytes, 24 for W = 5 and the pattern-database search
     g.smem = SearchSmem<W, PDB>::TABLES + (size_t)wpb * S * WarpStack<W, (W == 5) || PDB>::ENTRY_BYTES;
     // one kernel serves every block size (and the serving path), so its
     // dynamic shared memory limit is set once to the device's maximum; the
     // blocks per SM are looked up once per (device, block size, kernel)
     static std::map<std::tuple<int, int, int>, int> smem_limit;
-    int &lim = smem_limit[std::make_tuple(dev, cfg.variant, fuse ? 1 : 0)];
+    int &lim = smem_limit[std::make_tuple(dev, cfg.variant, form)];
     if (lim == 0) {
         // the device maximum less the kernel's static shared memory
         int optin = 0;
         cudaFuncAttributes fa;
         CK(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-        CK(cudaFuncGetAttributes(&fa, search_kernel<W, S, PDB>(cfg.variant, fuse)));
+        CK(cudaFuncGetAttributes(&fa, search_kernel<W, S, PDB>(cfg.variant, fuse, g.chain)));
         lim = optin - (int)fa.sharedSizeBytes;
-        CK(cudaFuncSetAttribute(search_kernel<W, S, PDB>(cfg.variant, fuse), cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
+        CK(cudaFuncSetAttribute(search_kernel<W, S, PDB>(cfg.variant, fuse, g.chain), cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
     }
     if (g.smem > (size_t)lim)
         return BPIDA_EINVAL;
+    int cap = 0;
+    if (g.chain) {
+        cap = chain_entries(wpb, (size_t)lim);
+        g.smem = Chain::BYTES + (size_t)wpb * ChainStack::bytes(cap);
+    }
     static std::map<std::tuple<int, int, int, int>, int> occ;
-    int &bpsm = occ[std::make_tuple(dev, wpb, cfg.variant, fuse ? 1 : 0)];
+    int &bpsm = occ[std::make_tuple(dev, wpb, cfg.variant, form)];
     if (bpsm == 0)
-        CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bpsm, search_kernel<W, S, PDB>(cfg.variant, fuse), g.threads, g.smem));
+        CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bpsm, search_kernel<W, S, PDB>(cfg.variant, fuse, g.chain), g.threads, g.smem));
     if (bpsm < 1)
         return BPIDA_EINVAL;
     g.grid = sms * bpsm;
@@ -433,8 +464,9 @@ bpida_status run(const Settings &cfg, const uint64_t *boards, int n, int *out_le
     // per-warp overflow stacks, and the hand-back queue: every warp's shared
     // and overflow stacks plus its unfinished chunk, twice over; overflowing
     // it is detected and reported as BPIDA_ENOMEM
-    const int ovf_cap = (W == 5) ? 4 * S : 0;
-    g.Q = std::max({(size_t)n * g.C, (size_t)g.total_warps * (S + ovf_cap + 32) * 2, (size_t)1 << 24}) + 1024;
+    const int ovf_cap = (W == 5) ? 4 * S : g.chain ? CHAIN_OVERFLOW : 0;
+    g.Q = std::max({(size_t)n * g.C, (size_t)g.total_warps * (std::max(S, 32 * cap + 32) + ovf_cap + 32) * 2,
+                    (size_t)1 << 24}) + 1024;
     if (g.Q > (size_t)INT_MAX / 2 || (size_t)n * 2 * g.C > (size_t)UINT32_MAX)
         return BPIDA_ENOMEM;
 
@@ -476,6 +508,7 @@ bpida_status run(const Settings &cfg, const uint64_t *boards, int n, int *out_le
     d.Q = (int)g.Q;
     d.ovf = (unsigned char *)ws.ovf.p;
     d.ovf_cap = ovf_cap;
+    d.chain_cap = cap;
     if (fuse) {
         char *p = (char *)ws.fuse.p;
         d.fuse.low = (unsigned long long *)p;
@@ -593,7 +626,7 @@ bpida_status run(const Settings &cfg, const uint64_t *boards, int n, int *out_le
         for (;;) {
             if (g_timing)
                 CK(cudaEventRecord(ws.ev0, st));
-            search_kernel<W, S, PDB>(cfg.variant, fuse)<<<g.grid, g.threads, g.smem, st>>>(d);
+            search_kernel<W, S, PDB>(cfg.variant, fuse, g.chain)<<<g.grid, g.threads, g.smem, st>>>(d);
             CK(cudaGetLastError());
             if (g_timing)
                 CK(cudaEventRecord(ws.ev1, st));

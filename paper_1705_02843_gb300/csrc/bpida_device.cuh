@@ -426,6 +426,7 @@ template <int W> struct Dev {
     unsigned *done_list;        // serving: instances that finished in this step (else null)
     unsigned char *ovf;         // per-warp overflow stacks in global memory (may be null)
     int ovf_cap;                // entries per warp overflow stack (0 = none)
+    int chain_cap;              // k_search_chain: stack entries per lane
     Fuse fuse;                  // fused iterations (fuse.jump null: one iteration per step)
     // Serving with time slices (slice = 1): an instance's iteration may run
     // over several steps. Frontier regions then belong to instance slots, not

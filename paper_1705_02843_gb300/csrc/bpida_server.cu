@@ -17,7 +17,7 @@
 // by the frontier memory the caller grants (each slot owns 2*C frontier
 // records), so admission is by frontier memory.
 #include "bpida.h"
-#include "bpida_device.cuh"
+#include "bpida_chain.cuh"
 
 #include <algorithm>
 #include <atomic>
@@ -35,7 +35,7 @@ using namespace bp;
 namespace {
 
 constexpr int SV_W = 4;
-constexpr int SV_S = 384;
+constexpr int SV_CAP = 20;  // search stack entries per lane
 constexpr int SV_WPB = 4;
 constexpr int SV_MAXLEN = Geo<SV_W>::MAXLEN;
 constexpr int SV_MAXIT = Geo<SV_W>::MAXIT;
@@ -150,7 +150,7 @@ bool bpida_server::device_step(int admitted)
         k_split<SV_W><<<n_active, SPLIT_THREADS, 0, st>>>(d);
         SV_CK(cudaGetLastError());
         for (;;) {
-            k_search<SV_W, SV_S><<<grid, threads, smem, st>>>(d);
+            k_search_chain<><<<grid, threads, smem, st>>>(d);
             SV_CK(cudaGetLastError());
             SV_CK(cudaMemcpyAsync(h_ctrl, d.ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, st));
             SV_CK(cudaStreamSynchronize(st));
@@ -287,16 +287,16 @@ bpida_server *bpida_server_create(const bpida_config *cfg, size_t frontier_bytes
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, sv->dev);
     sv->max_slots = slots;
     sv->threads = SV_WPB * 32;
-    sv->smem = SearchSmem<SV_W>::TABLES + (size_t)SV_WPB * SV_S * WarpStack<SV_W>::ENTRY_BYTES;
+    sv->smem = Chain::BYTES + (size_t)SV_WPB * ChainStack::bytes(SV_CAP);
     int bpsm = 0, smem_max = 0;
     // the device maximum, as the solve path sets it: the kernel is shared
     cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, sv->dev);
     cudaFuncAttributes fa;
-    if (cudaFuncGetAttributes(&fa, k_search<SV_W, SV_S>) == cudaSuccess)
+    if (cudaFuncGetAttributes(&fa, k_search_chain<>) == cudaSuccess)
         smem_max -= (int)fa.sharedSizeBytes;  // less the kernel's static shared memory
-    if (cudaFuncSetAttribute(k_search<SV_W, SV_S>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max) !=
+    if (cudaFuncSetAttribute(k_search_chain<>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max) !=
             cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bpsm, k_search<SV_W, SV_S>, sv->threads, sv->smem) !=
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bpsm, k_search_chain<>, sv->threads, sv->smem) !=
             cudaSuccess ||
         bpsm < 1) {
         delete sv;
@@ -304,8 +304,8 @@ bpida_server *bpida_server_create(const bpida_config *cfg, size_t frontier_bytes
     }
     sv->grid = sms * bpsm;
     const int total_warps = sv->grid * SV_WPB;
-    const int ovf_cap = 0;  // 15-puzzle: no overflow stacks
-    const size_t Q = std::max({(size_t)slots * C, (size_t)total_warps * (SV_S + ovf_cap + 32) * 2, (size_t)1 << 24}) + 1024;
+    const int ovf_cap = CHAIN_OVERFLOW;
+    const size_t Q = std::max({(size_t)slots * C, (size_t)total_warps * (32 * SV_CAP + 32 + ovf_cap + 32) * 2, (size_t)1 << 24}) + 1024;
 
     // one allocation carved into the workspace
     const size_t n = (size_t)slots;
@@ -346,6 +346,7 @@ bpida_server *bpida_server_create(const bpida_config *cfg, size_t frontier_bytes
     d.Q = (int)Q;
     d.ovf = (unsigned char *)(b + o_ovf);
     d.ovf_cap = ovf_cap;
+    d.chain_cap = SV_CAP;
     d.slice = 1;
     d.carry = (unsigned *)(b + o_carry);
     d.fbase = (int *)(b + o_fbase);
