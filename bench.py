@@ -69,20 +69,20 @@ WORKLOAD_DESC = {
 # 2 cycles, so above one half the ALU pipe, not issue, bounds the kernel at
 # issue peak / (2 x share)), and DRAM bytes (read + write) of the captured
 # launch, for the kernel each form runs.
-#   batched: k_search<4,384,0>, a steady-state launch (the first pass of a
-#   step, hand-back on) of a batched solve of the 4096-board mix: 331.2 M
-#   warp instructions over 77.2 M nodes; ALU share (issue 84.0 %, ALU pipe
-#   64.9 % busy) and DRAM bytes from one full capture of such a launch
-#   (profiles/k_search_15puzzle_mixed15_4096_batched.txt). Hand-back passes
-#   with few nodes issue more per node (4.4-5.4), so issue utilisation
-#   computed with this figure is a lower bound;
+#   batched: k_search_chain, a launch of 3.0e8 nodes of a batched solve of 12
+#   random permutations: 798.3 M warp instructions; ALU share (issue 70.6 %,
+#   ALU pipe 73.5 % busy) from the same capture
+#   (profiles/k_search_chain_15puzzle_perms_batched.txt). DRAM bytes from a
+#   full capture of the four-move kernel on the 4096-board mix
+#   (profiles/k_search_15puzzle_mixed15_4096_batched.txt): frontier records,
+#   queue and counters, the same in both;
 #   plain: the fused-iteration variant k_search<4,384,1>, the final iteration
 #   of board 0 of the mix as one pass
 #   (profiles/k_search_15puzzle_plain_fused_final_iteration.txt); its ALU
 #   share is the batched kernel's (the same step; a single-board launch's
 #   pipe fractions are skewed by its tail).
 KERNEL_COUNTERS = {
-    "batched": {"kernel": "k_search<4,384,0>", "instr_per_expansion": 4.29, "alu_pipe_share": 0.386,
+    "batched": {"kernel": "k_search_chain<96>", "instr_per_expansion": 2.65, "alu_pipe_share": 0.52,
                 "traffic_per_launch": 10233088},
     "plain": {"kernel": "k_search<4,384,1>", "instr_per_expansion": 4.66, "alu_pipe_share": 0.386,
               "traffic_per_launch": None},

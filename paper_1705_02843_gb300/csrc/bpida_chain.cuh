@@ -169,7 +169,10 @@ struct ChainStack {
         put_if(1u, to, x, y, z, w);
     }
 };
-static constexpr int CHAIN_OVERFLOW = 512;  // entries of a warp's overflow stack in global memory
+// Entries of a warp's overflow stack in global memory: about the open nodes of 32
+// paths of the deepest searches. With 512 the hand-back queue overflowed on a
+// batch with a board of more than 1e11 nodes.
+static constexpr int CHAIN_OVERFLOW = 4096;
 
 // Chain step: the records a warp works on, consecutive records of one
 // instance in the pass's input: src[i] is record i.

@@ -46,3 +46,20 @@ def test_first_solution_and_budget():
             assert (g["status"], g["nodes"], g["solutions"]) == (0, r["nodes"], r["solutions"])
         else:
             assert g["status"] == bpida.EBUDGET and g["nodes"] == r["nodes"][:len(g["nodes"])]
+
+
+def test_very_hard_batch_stays_within_the_queues():
+    """A batch whose hardest board expands more than 1e11 nodes: every board
+    ends with its result, the same as in calls of k_search's size."""
+    rng = I.Xoshiro256ss(0x5EED0000 + 31)
+    tiles = []
+    for _ in range(100):
+        s = rng.next_u64()
+        rng.below(100)
+        tiles.append(I.make_perm(4, s).tiles)
+    rc, got = gpu_solve(4, tiles)
+    assert rc == bpida.OK
+    halves = gpu_solve(4, tiles[:50])[1] + gpu_solve(4, tiles[50:])[1]
+    for g, h in zip(got, halves):
+        assert g["status"] == h["status"] == bpida.OK
+        assert (g["length"], g["nodes"], g["moves"], g["solutions"]) == (h["length"], h["nodes"], h["moves"], h["solutions"])
