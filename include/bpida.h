@@ -102,7 +102,10 @@ typedef struct {
                              384, 480, 512, 768, 1024. Smaller stacks
                              spill to the hand-back queue more often: with
                              256 a batch of hard boards can overflow it
-                             (those instances end with BPIDA_ENOMEM) */
+                             (those instances end with BPIDA_ENOMEM).
+                             The large steps of 15-puzzle calls of at
+                             least 64 boards (bpida_get_chain_passes)
+                             have stacks of a fixed size instead */
     int exit_fraction_pct;/* percentage of warps that must have run out of
                              work before busy warps hand their stacks back
                              for redistribution; 0 = auto */
@@ -330,6 +333,11 @@ void bpida_server_destroy(bpida_server *sv);
  * CUDA events on the launching stream (driver = 1 only). */
 void bpida_set_timing(int on);
 void bpida_get_stats(bpida_stats *out);
+/* Of bpida_stats.passes, the search passes that ran the kernel of large
+ * steps (15-puzzle calls of at least 64 boards with variant 0: steps predicted
+ * to expand 3e8 nodes or more; the other steps run the kernel of smaller
+ * calls). Complete when bpida_get_stats is. */
+uint64_t bpida_get_chain_passes(void);
 /* The search kernel launches of this host thread's last solve call, if it
  * ran the host-driven loop (driver = 1) with timing on: launch i took ms[i]
  * milliseconds (CUDA events on the launching stream) and popped nodes[i]

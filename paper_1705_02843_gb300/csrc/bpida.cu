@@ -5,7 +5,8 @@
 // f-limited iteration of every still-active instance (each at its own
 // limit), or several consecutive ones searched together (fused iterations,
 // calls of a few boards): k_split builds each instance's root set (its last
-// block computes the frontier offsets), k_search passes consume the
+// block computes the frontier offsets), k_search passes (in large steps of
+// 15-puzzle calls of many boards: k_search_chain passes) consume the
 // frontiers with persistent warps (another pass only when warps handed work
 // back; the last block of a pass decides), and k_advance records the
 // iterations' node counts and raises each limit to the smallest pruned f,
@@ -56,6 +57,7 @@ struct LaunchRec {
     uint64_t nodes;
 };
 thread_local std::vector<LaunchRec> g_launch_log;
+thread_local uint64_t g_chain_passes = 0;  // of this thread's last host-driven call
 std::atomic<unsigned long long> g_fuse_nodes{0};  // 0: the defaults below
 std::mutex g_mu;
 
@@ -298,17 +300,19 @@ struct Geometry {
     int n_cap;
     int variant;
     bool fuse;
-    int chain;  // k_search_chain: its warps per block, else 0
 };
 
-// 15-puzzle calls of at least CHAIN_MIN_N boards search with k_search_chain.
-// It is the faster one wherever the search itself is the time (random
-// permutations: 64 boards 229.7 ms against 300.4 with k_search, 16 boards 42.0
-// against 51.9), and the slower one on short searches, whose time is how soon
-// a record spreads over a warp's lanes (40-move walks: 16 boards 1150 us
-// against 1050, 64 boards 1686 against 1546). The number of boards does not
-// tell the two apart; the line lies where a batch is more likely to hold a
-// hard board, and below it easy small calls keep the shorter time.
+// k_search_chain's launch: stack entries per lane (0: the call does not use it)
+struct ChainGeometry {
+    int cap, grid, total_warps;
+    size_t smem;
+};
+
+// 15-puzzle calls of at least CHAIN_MIN_N boards search their large steps
+// (CHAIN_MIN_NODES, bpida_chain.cuh) with k_search_chain, in a pass loop of
+// its own. Smaller calls are without that loop: skipping it takes about 1 % of
+// a call of easy boards (64 40-move walks 1471 us; 63 of them, without it,
+// 1449).
 constexpr int CHAIN_MIN_N = 64;
 // Its stack entries per lane: 20 where they fit (five 4-warp blocks per SM;
 // every block size that a caller can ask for leaves room for 13).
@@ -319,15 +323,45 @@ int chain_entries(int wpb, size_t lim)
         --cap;
     return cap;
 }
+void (*chain_kernel(int wpb))(const Dev<4>) { return wpb > CHAIN_WARPS ? k_search_chain<64> : k_search_chain<>; }
+
+// k_search_chain's launch with blocks of wpb warps, looked up once per
+// (device, block size).
+cudaError_t chain_geometry(int dev, int sms, int wpb, ChainGeometry &gc)
+{
+    static std::map<std::pair<int, int>, std::pair<int, int>> known;  // entries per lane, blocks per SM
+    auto &k = known[std::make_pair(dev, wpb)];
+    if (k.second == 0) {
+        int optin = 0;
+        cudaFuncAttributes fa;
+        cudaError_t e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+        if (e == cudaSuccess)
+            e = cudaFuncGetAttributes(&fa, chain_kernel(wpb));
+        if (e != cudaSuccess)
+            return e;
+        const int lim = optin - (int)fa.sharedSizeBytes;  // less the kernel's static shared memory
+        if ((e = cudaFuncSetAttribute(chain_kernel(wpb), cudaFuncAttributeMaxDynamicSharedMemorySize, lim)) != cudaSuccess)
+            return e;
+        k.first = chain_entries(wpb, (size_t)lim);
+        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&k.second, chain_kernel(wpb), wpb * 32,
+                                                               Chain::BYTES + (size_t)wpb * ChainStack::bytes(k.first))) !=
+            cudaSuccess)
+            return e;
+        if (k.second < 1)
+            return cudaErrorInvalidConfiguration;
+    }
+    gc.cap = k.first;
+    gc.grid = sms * k.second;
+    gc.total_warps = gc.grid * wpb;
+    gc.smem = Chain::BYTES + (size_t)wpb * ChainStack::bytes(k.first);
+    return cudaSuccess;
+}
 
 // variant 0: warp per subtree group; 1: the paper's kernel; 6: block per
 // subtree group (the autotuner's other mode, widths 3 and 4)
 constexpr int VARIANT_BLOCK = 6;
-template <int W, int S, bool PDB> void (*search_kernel(int variant, bool fuse, int chain))(const Dev<W>)
+template <int W, int S, bool PDB> void (*search_kernel(int variant, bool fuse))(const Dev<W>)
 {
-    if constexpr (W == 4 && !PDB)
-        if (chain)
-            return chain > CHAIN_WARPS ? k_search_chain<64> : k_search_chain<>;
     if constexpr (PDB) {
         return fuse ? k_search<W, S, true, true> : k_search<W, S, false, true>;
     } else {
@@ -352,8 +386,12 @@ int split_threads(int n) { return n >= SPLIT_SMALL_N ? SPLIT_THREADS_SMALL : SPL
 
 // The whole solve as one graph (k_set_desc is launched before it):
 //   init -> WHILE(step){ split -> WHILE(pass){ search } -> advance } -> finalize
+// d_chain: the same as d with k_search_chain's limits; where the call uses that
+// kernel (gc.cap), the step has a second pass loop, and the splitter starts
+// one of the two.
 template <int W, int S, bool PDB>
-cudaError_t build_graph(Plan &pl, Dev<W> d, const Geometry &g, const char **where)
+cudaError_t build_graph(Plan &pl, Dev<W> d, const Geometry &g, const Dev<W> &d_chain, const ChainGeometry &gc,
+                        const char **where)
 {
     cudaGraph_t G;
     *where = "cudaGraphCreate";
@@ -368,6 +406,7 @@ cudaError_t build_graph(Plan &pl, Dev<W> d, const Geometry &g, const char **wher
     d.graph = 1;
     d.h_step = hs;
     d.h_pass = 0;
+    d.h_chain = 0;
     const dim3 b128(128);
     const dim3 g_inst((g.n_cap + 127) / 128), g_prob(g.n_cap);
     cudaGraphNode_t n_init, n_step, n_fin;
@@ -384,6 +423,12 @@ cudaError_t build_graph(Plan &pl, Dev<W> d, const Geometry &g, const char **wher
     if ((e = cudaGraphConditionalHandleCreate(&hp, B, 0, cudaGraphCondAssignDefault)) != cudaSuccess)
         return e;
     d.h_pass = hp;
+    if (gc.cap) {
+        cudaGraphConditionalHandle hc;
+        if ((e = cudaGraphConditionalHandleCreate(&hc, B, 0, cudaGraphCondAssignDefault)) != cudaSuccess)
+            return e;
+        d.h_chain = hc;
+    }
     cudaGraphNode_t n_split, n_pass, n_adv;
     *where = "split/pass/advance nodes";
     if ((e = add_kernel(&n_split, B, nullptr, 0, split_kernel<W, PDB>(g.n_cap), g_prob, dim3(split_threads(g.n_cap)), 0, d)) != cudaSuccess)
@@ -391,12 +436,26 @@ cudaError_t build_graph(Plan &pl, Dev<W> d, const Geometry &g, const char **wher
     cudaGraph_t P;
     if ((e = add_while(&n_pass, B, &n_split, 1, hp, &P)) != cudaSuccess)
         return e;
+    if constexpr (W == 4 && !PDB)
+        if (gc.cap) {
+            cudaGraph_t PC;
+            cudaGraphNode_t n_chain, n_loop = n_pass;
+            Dev<W> dc = d_chain;
+            dc.graph = 1;
+            dc.h_step = hs;
+            dc.h_pass = d.h_chain;
+            if ((e = add_while(&n_pass, B, &n_loop, 1, d.h_chain, &PC)) != cudaSuccess)
+                return e;
+            if ((e = add_kernel(&n_chain, PC, nullptr, 0, chain_kernel(g.threads / 32), dim3(gc.grid), dim3(g.threads), gc.smem,
+                                dc)) != cudaSuccess)
+                return e;
+        }
     if ((e = add_kernel(&n_adv, B, &n_pass, 1, k_advance<W>, g_inst, b128, 0, d)) != cudaSuccess)
         return e;
 
     cudaGraphNode_t n_search;
     *where = "search node";
-    if ((e = add_kernel(&n_search, P, nullptr, 0, search_kernel<W, S, PDB>(g.variant, g.fuse, g.chain), dim3(g.grid), dim3(g.threads),
+    if ((e = add_kernel(&n_search, P, nullptr, 0, search_kernel<W, S, PDB>(g.variant, g.fuse), dim3(g.grid), dim3(g.threads),
                         g.smem, d)) != cudaSuccess)
         return e;
     *where = "cudaGraphInstantiate";
@@ -426,47 +485,43 @@ bpida_status run(const Settings &cfg, const uint64_t *boards, int n, int *out_le
     g.fuse = fuse;
     const int wpb = cfg.variant == 1 ? 1 : cfg.wpb;  // the paper's kernel: block = warp
     g.threads = wpb * 32;
-    g.chain = (W == 4 && !PDB && cfg.variant == 0 && n >= CHAIN_MIN_N) ? wpb : 0;
-    const int form = (fuse ? 1 : 0) + (g.chain ? (wpb > CHAIN_WARPS ? 4 : 2) : 0);
     // search stack entries: 16 bytes, 24 for W = 5 and the pattern-database search
     g.smem = SearchSmem<W, PDB>::TABLES + (size_t)wpb * S * WarpStack<W, (W == 5) || PDB>::ENTRY_BYTES;
-    // one kernel serves every block size (and the serving path), so its
+    // one kernel serves every block size, so its
     // dynamic shared memory limit is set once to the device's maximum; the
     // blocks per SM are looked up once per (device, block size, kernel)
     static std::map<std::tuple<int, int, int>, int> smem_limit;
-    int &lim = smem_limit[std::make_tuple(dev, cfg.variant, form)];
+    int &lim = smem_limit[std::make_tuple(dev, cfg.variant, fuse ? 1 : 0)];
     if (lim == 0) {
         // the device maximum less the kernel's static shared memory
         int optin = 0;
         cudaFuncAttributes fa;
         CK(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-        CK(cudaFuncGetAttributes(&fa, search_kernel<W, S, PDB>(cfg.variant, fuse, g.chain)));
+        CK(cudaFuncGetAttributes(&fa, search_kernel<W, S, PDB>(cfg.variant, fuse)));
         lim = optin - (int)fa.sharedSizeBytes;
-        CK(cudaFuncSetAttribute(search_kernel<W, S, PDB>(cfg.variant, fuse, g.chain), cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
+        CK(cudaFuncSetAttribute(search_kernel<W, S, PDB>(cfg.variant, fuse), cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
     }
     if (g.smem > (size_t)lim)
         return BPIDA_EINVAL;
-    int cap = 0;
-    if (g.chain) {
-        cap = chain_entries(wpb, (size_t)lim);
-        g.smem = Chain::BYTES + (size_t)wpb * ChainStack::bytes(cap);
-    }
     static std::map<std::tuple<int, int, int, int>, int> occ;
-    int &bpsm = occ[std::make_tuple(dev, wpb, cfg.variant, form)];
+    int &bpsm = occ[std::make_tuple(dev, wpb, cfg.variant, fuse ? 1 : 0)];
     if (bpsm == 0)
-        CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bpsm, search_kernel<W, S, PDB>(cfg.variant, fuse, g.chain), g.threads, g.smem));
+        CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bpsm, search_kernel<W, S, PDB>(cfg.variant, fuse), g.threads, g.smem));
     if (bpsm < 1)
         return BPIDA_EINVAL;
     g.grid = sms * bpsm;
     g.total_warps = g.grid * wpb;
+    ChainGeometry gc = {0, 0, 0, 0};
+    if (W == 4 && !PDB && cfg.variant == 0 && n >= CHAIN_MIN_N)
+        CK(chain_geometry(dev, sms, wpb, gc));
     g.tcap = cfg.split_target > 0 ? cfg.split_target : std::max(2, std::min(4096, (1 << 21) / std::max(n, 1)));
     g.C = 4 * g.tcap + 4;
     // per-warp overflow stacks, and the hand-back queue: every warp's shared
     // and overflow stacks plus its unfinished chunk, twice over; overflowing
     // it is detected and reported as BPIDA_ENOMEM
-    const int ovf_cap = (W == 5) ? 4 * S : g.chain ? CHAIN_OVERFLOW : 0;
-    g.Q = std::max({(size_t)n * g.C, (size_t)g.total_warps * (std::max(S, 32 * cap + 32) + ovf_cap + 32) * 2,
-                    (size_t)1 << 24}) + 1024;
+    const int ovf_cap = (W == 5) ? 4 * S : gc.cap ? CHAIN_OVERFLOW : 0;
+    g.Q = std::max({(size_t)n * g.C, (size_t)g.total_warps * (S + (gc.cap ? 0 : ovf_cap) + 32) * 2,
+                    (size_t)gc.total_warps * (32 * gc.cap + 32 + ovf_cap + 32) * 2, (size_t)1 << 24}) + 1024;
     if (g.Q > (size_t)INT_MAX / 2 || (size_t)n * 2 * g.C > (size_t)UINT32_MAX)
         return BPIDA_ENOMEM;
 
@@ -481,7 +536,7 @@ bpida_status run(const Settings &cfg, const uint64_t *boards, int n, int *out_le
     CK(ws.ensure(ws.q1, sizeof(Rec<W>) * g.Q));
     CK(ws.ensure(ws.ctrl, sizeof(Ctrl)));
     CK(ws.ensure(ws.desc, sizeof(CallDesc)));
-    CK(ws.ensure(ws.ovf, (size_t)g.total_warps * ovf_cap * WarpStack<W>::ENTRY_BYTES));
+    CK(ws.ensure(ws.ovf, (size_t)(gc.cap ? gc.total_warps : g.total_warps) * ovf_cap * WarpStack<W>::ENTRY_BYTES));
     if (fuse)
         CK(ws.ensure(ws.fuse, (size_t)n * (sizeof(int) + FUSE_K * (2 * sizeof(unsigned long long) + sizeof(unsigned)))));
     if (!ws.h_ctrl)
@@ -508,7 +563,7 @@ bpida_status run(const Settings &cfg, const uint64_t *boards, int n, int *out_le
     d.Q = (int)g.Q;
     d.ovf = (unsigned char *)ws.ovf.p;
     d.ovf_cap = ovf_cap;
-    d.chain_cap = cap;
+    d.chain_cap = gc.cap;
     if (fuse) {
         char *p = (char *)ws.fuse.p;
         d.fuse.low = (unsigned long long *)p;
@@ -544,6 +599,7 @@ bpida_status run(const Settings &cfg, const uint64_t *boards, int n, int *out_le
     d.tune.target_path = std::min(g.tcap, 4096);
     d.tune.growth = 8;
     d.tune.min_pass_ns = cfg.min_pass_ns;
+    d.tune.chain_nodes = gc.cap ? CHAIN_MIN_NODES : 0ull;
     d.lut = make_move_lut<W>();
     if constexpr (PDB) {
         d.pdb.tab = cfg.pdb->tab;
@@ -551,6 +607,8 @@ bpida_status run(const Settings &cfg, const uint64_t *boards, int n, int *out_le
         d.pdb.goal = cfg.pdb->goal;
         d.pdb.goal_sb = cfg.pdb->goal_sb;
     }
+    Dev<W> dc = d;
+    dc.tune.exit_threshold = std::max(1, (int)((long long)gc.total_warps * cfg.exit_pct / 100));
 
     CallDesc desc;
     std::memset(&desc, 0, sizeof desc);
@@ -583,7 +641,7 @@ bpida_status run(const Settings &cfg, const uint64_t *boards, int n, int *out_le
             ws.trim_plans();
             Plan &pl = ws.plans[key];
             const char *where = "";
-            cudaError_t e = build_graph<W, S, PDB>(pl, d, g, &where);
+            cudaError_t e = build_graph<W, S, PDB>(pl, d, g, dc, gc, &where);
             if (e != cudaSuccess) {
                 std::fprintf(stderr, "bpida: graph build failed at %s: %s\n", where, cudaGetErrorString(e));
                 pl.destroy();
@@ -626,7 +684,15 @@ bpida_status run(const Settings &cfg, const uint64_t *boards, int n, int *out_le
         for (;;) {
             if (g_timing)
                 CK(cudaEventRecord(ws.ev0, st));
-            search_kernel<W, S, PDB>(cfg.variant, fuse, g.chain)<<<g.grid, g.threads, g.smem, st>>>(d);
+            // (h_ctrl: read back after k_init or k_advance, which set chain)
+            if constexpr (W == 4 && !PDB) {
+                if (gc.cap && ws.h_ctrl->chain)
+                    chain_kernel(wpb)<<<gc.grid, g.threads, gc.smem, st>>>(dc);
+                else
+                    search_kernel<W, S, PDB>(cfg.variant, fuse)<<<g.grid, g.threads, g.smem, st>>>(d);
+            } else {
+                search_kernel<W, S, PDB>(cfg.variant, fuse)<<<g.grid, g.threads, g.smem, st>>>(d);
+            }
             CK(cudaGetLastError());
             if (g_timing)
                 CK(cudaEventRecord(ws.ev1, st));
@@ -660,6 +726,7 @@ bpida_status run(const Settings &cfg, const uint64_t *boards, int n, int *out_le
     ws.last_call = ++g_calls;
     CK(cudaStreamSynchronize(st));
     fill_loop_stats(stats, *ws.h_ctrl, false);
+    g_chain_passes = ws.h_ctrl->chain_passes;
     g_stats = stats;
     g_last.ws = nullptr;
     const Ctrl &c = *ws.h_ctrl;
@@ -877,6 +944,14 @@ int bpida_get_launch_log(double *ms, uint64_t *nodes, int cap)
             nodes[i] = g_launch_log[i].nodes;
     }
     return k;
+}
+
+uint64_t bpida_get_chain_passes(void)
+{
+    if (!g_last.ws)
+        return g_chain_passes;
+    std::lock_guard<std::mutex> lock(g_mu);
+    return g_last.ws->last_call == g_last.call && g_last.ws->h_ctrl ? g_last.ws->h_ctrl->chain_passes : 0;
 }
 
 void bpida_set_fuse_nodes(uint64_t nodes) { g_fuse_nodes.store(nodes); }

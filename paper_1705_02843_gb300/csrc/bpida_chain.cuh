@@ -1,7 +1,7 @@
-// The 15-puzzle's Manhattan search for large work: calls of many boards and
-// the serving loop (k_search_chain). Calls of a few boards run k_search's
-// four-move step (bpida_device.cuh): its warps share one stack, so that the
-// short runs of a small call spread over a warp's lanes sooner.
+// The 15-puzzle's Manhattan search for large work: the large steps of calls
+// of many boards and of the serving loop (k_search_chain). Short steps run
+// k_search's four-move step (bpida_device.cuh): its warps share one stack, so
+// that their short runs spread over a warp's lanes sooner.
 //
 // Nothing here waits on another warp, block or kernel: every loop is bounded
 // by the work it consumes.
@@ -173,6 +173,20 @@ struct ChainStack {
 // paths of the deepest searches. With 512 the hand-back queue overflowed on a
 // batch with a board of more than 1e11 nodes.
 static constexpr int CHAIN_OVERFLOW = 4096;
+
+// A step searches with this kernel when it is predicted to expand at least
+// CHAIN_MIN_NODES nodes (k_advance's sum over the step's instances, eight
+// times their last iterations), else with k_search: this one is the faster
+// one where the search itself is the time, and the slower one on short
+// searches, whose time is how soon a record spreads over a warp's lanes. Both
+// sides measured, k_search in every step / this kernel in every step / the
+// rule: 512 40-move walks 2443 / 2787 / 2443 us, 64 50-to-60-move walks 2559 /
+// 2893 / 2562 us, 700 of them 12.52 / 12.02 / 11.84 ms, 300 boards with 1 %
+// permutations 13.07 / 12.54 / 12.36 ms, 100 permutations 430.9 / 327.9 /
+// 327.7 ms; the service, 1000 30-to-50-move walks at once 8.54 / 8.93 / 8.48
+// ms. The line is flat from 1e8 (walks of 40 moves, 4096 at once: 6.31 ms
+// against 6.06) to 1e9 (the 700 walks: 12.13 ms).
+static constexpr unsigned long long CHAIN_MIN_NODES = 300000000ull;
 
 // Chain step: the records a warp works on, consecutive records of one
 // instance in the pass's input: src[i] is record i.
@@ -660,6 +674,7 @@ __global__ void __maxnreg__(REGS) k_search_chain(const Dev<4> a)
             __threadfence();
             if (atomicAdd(&a.ctrl->done_warps, 1) == (int)gridDim.x - 1) {
                 __threadfence();
+                a.ctrl->chain_passes += 1;
                 end_of_pass<W>(a);
             }
         }

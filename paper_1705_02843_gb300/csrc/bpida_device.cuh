@@ -221,6 +221,9 @@ struct Ctrl {
     unsigned long long passes_total;
     unsigned long long search_ns;           // sum of k_search durations (globaltimer)
     unsigned long long t_start, t_end;      // this pass's first block start / last block end
+    unsigned long long pred;                // nodes that the next step is predicted to expand (k_advance's sum)
+    unsigned long long chain_passes;        // search passes of k_search_chain
+    int chain;                              // 1: this step searches with k_search_chain
 };
 static constexpr int MAX_STEPS = 100000;        // loop guards: exceeding one is an
 static constexpr int MAX_PASSES_PER_STEP = 100000;  // internal error, never a hang
@@ -350,6 +353,7 @@ struct Tune {
     int growth;          // expected node growth per iteration (x)
     int min_pass_ns;     // a pass hands work back only after running this long
     unsigned long long step_ns;  // serving: time slice of a step (0 = none)
+    unsigned long long chain_nodes;  // predicted nodes from which a step searches with k_search_chain (0: never)
 };
 
 // ---------------------------------------------------------------------
@@ -422,6 +426,7 @@ template <int W> struct Dev {
     Tune tune;
     MoveLut<W> lut;
     cudaGraphConditionalHandle h_step, h_pass;
+    cudaGraphConditionalHandle h_chain;  // the pass loop of steps that search with k_search_chain
     int graph;                  // 1 inside the CUDA graph (sets the loop conditions)
     unsigned *done_list;        // serving: instances that finished in this step (else null)
     unsigned char *ovf;         // per-warp overflow stacks in global memory (may be null)
@@ -2352,7 +2357,7 @@ __global__ void __launch_bounds__(SMALLB ? SPLIT_THREADS_SMALL : SPLIT_THREADS) 
         ctrl->records_total += (unsigned long long)n_front;
         __threadfence();
         if (a.graph)
-            cudaGraphSetConditional(a.h_pass, 1u);
+            cudaGraphSetConditional(ctrl->chain ? a.h_chain : a.h_pass, 1u);
     }
 }
 
@@ -2548,6 +2553,8 @@ __global__ void k_advance(const Dev<W> a)
                     want = want < 1ull ? 1ull : want;
                     want = want > (unsigned long long)a.tune.target_cap ? (unsigned long long)a.tune.target_cap : want;
                     st.target = (uint32_t)want;
+                    if (a.tune.chain_nodes)
+                        atomicAdd(&ctrl->pred, pred);
                 }
             }
         } else if (st.mode == MODE_PATH) {
@@ -2578,6 +2585,12 @@ __global__ void k_advance(const Dev<W> a)
         c->steps += 1;
         if (c->steps >= MAX_STEPS)
             c->err |= ERR_INTERNAL;
+        // the next step's search kernel (path steps, whose subtrees are small,
+        // predict nothing); open nodes carried over a time slice are
+        // k_search_chain's to continue: only it reads its own records
+        c->chain = a.tune.chain_nodes != 0ull &&
+                   (*(volatile unsigned long long *)&c->pred >= a.tune.chain_nodes || c->n_carry > 0);
+        c->pred = 0;
         c->step_again = (c->n_active > 0 && *(volatile int *)&c->err == 0) ? 1 : 0;
         __threadfence();
         if (a.graph)

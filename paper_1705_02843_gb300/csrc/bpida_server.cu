@@ -35,7 +35,8 @@ using namespace bp;
 namespace {
 
 constexpr int SV_W = 4;
-constexpr int SV_CAP = 20;  // search stack entries per lane
+constexpr int SV_S = 384;   // k_search: stack entries per warp
+constexpr int SV_CAP = 20;  // k_search_chain: stack entries per lane
 constexpr int SV_WPB = 4;
 constexpr int SV_MAXLEN = Geo<SV_W>::MAXLEN;
 constexpr int SV_MAXIT = Geo<SV_W>::MAXIT;
@@ -88,8 +89,9 @@ struct Req {
 struct bpida_server {
     int dev = 0;
     int max_slots = 0;
-    int grid = 0, threads = 0;
-    size_t smem = 0;
+    int grid = 0, chain_grid = 0, threads = 0;
+    int exit_threshold = 0, chain_exit_threshold = 0;
+    size_t smem = 0, chain_smem = 0;
     cudaStream_t st = nullptr;
     void *mem = nullptr;
     Dev<SV_W> d;
@@ -144,13 +146,18 @@ bool bpida_server::device_step(int admitted)
     SV_CK(cudaMemcpyAsync(h_ctrl, d.ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, st));
     SV_CK(cudaStreamSynchronize(st));
     const int n_active = h_ctrl->n_active;
+    const bool chain = h_ctrl->chain != 0;  // this step's search kernel (set by the last k_advance)
+    d.tune.exit_threshold = chain ? chain_exit_threshold : exit_threshold;
     uint64_t passes = 0, steps = 0, sliced = 0;
     d.tune.step_ns = (unsigned long long)std::max(0ll, slice_ns.load());
     if (n_active > 0) {
         k_split<SV_W><<<n_active, SPLIT_THREADS, 0, st>>>(d);
         SV_CK(cudaGetLastError());
         for (;;) {
-            k_search_chain<><<<grid, threads, smem, st>>>(d);
+            if (chain)
+                k_search_chain<><<<chain_grid, threads, chain_smem, st>>>(d);
+            else
+                k_search<SV_W, SV_S><<<grid, threads, smem, st>>>(d);
             SV_CK(cudaGetLastError());
             SV_CK(cudaMemcpyAsync(h_ctrl, d.ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, st));
             SV_CK(cudaStreamSynchronize(st));
@@ -287,25 +294,31 @@ bpida_server *bpida_server_create(const bpida_config *cfg, size_t frontier_bytes
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, sv->dev);
     sv->max_slots = slots;
     sv->threads = SV_WPB * 32;
-    sv->smem = Chain::BYTES + (size_t)SV_WPB * ChainStack::bytes(SV_CAP);
-    int bpsm = 0, smem_max = 0;
-    // the device maximum, as the solve path sets it: the kernel is shared
-    cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, sv->dev);
-    cudaFuncAttributes fa;
-    if (cudaFuncGetAttributes(&fa, k_search_chain<>) == cudaSuccess)
-        smem_max -= (int)fa.sharedSizeBytes;  // less the kernel's static shared memory
-    if (cudaFuncSetAttribute(k_search_chain<>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max) !=
-            cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bpsm, k_search_chain<>, sv->threads, sv->smem) !=
-            cudaSuccess ||
-        bpsm < 1) {
+    sv->smem = SearchSmem<SV_W>::TABLES + (size_t)SV_WPB * SV_S * WarpStack<SV_W>::ENTRY_BYTES;
+    sv->chain_smem = Chain::BYTES + (size_t)SV_WPB * ChainStack::bytes(SV_CAP);
+    // blocks per SM of a kernel; its dynamic shared memory limit goes to the
+    // device maximum, as the solve path sets it (the kernels are shared)
+    auto blocks_per_sm = [&](void (*kernel)(const Dev<SV_W>), size_t smem) -> int {
+        int bpsm = 0, smem_max = 0;
+        cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, sv->dev);
+        cudaFuncAttributes fa;
+        if (cudaFuncGetAttributes(&fa, kernel) == cudaSuccess)
+            smem_max -= (int)fa.sharedSizeBytes;  // less the kernel's static shared memory
+        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max) != cudaSuccess ||
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bpsm, kernel, sv->threads, smem) != cudaSuccess)
+            return 0;
+        return bpsm;
+    };
+    sv->grid = sms * blocks_per_sm(k_search<SV_W, SV_S>, sv->smem);
+    sv->chain_grid = sms * blocks_per_sm(k_search_chain<>, sv->chain_smem);
+    if (sv->grid < 1 || sv->chain_grid < 1) {
         delete sv;
         return nullptr;
     }
-    sv->grid = sms * bpsm;
-    const int total_warps = sv->grid * SV_WPB;
+    const int total_warps = sv->grid * SV_WPB, chain_warps = sv->chain_grid * SV_WPB;
     const int ovf_cap = CHAIN_OVERFLOW;
-    const size_t Q = std::max({(size_t)slots * C, (size_t)total_warps * (32 * SV_CAP + 32 + ovf_cap + 32) * 2, (size_t)1 << 24}) + 1024;
+    const size_t Q = std::max({(size_t)slots * C, (size_t)total_warps * (SV_S + 32) * 2,
+                               (size_t)chain_warps * (32 * SV_CAP + 32 + ovf_cap + 32) * 2, (size_t)1 << 24}) + 1024;
 
     // one allocation carved into the workspace
     const size_t n = (size_t)slots;
@@ -323,7 +336,7 @@ bpida_server *bpida_server_create(const bpida_config *cfg, size_t frontier_bytes
     const size_t o_done = take(4 * n), o_aslot = take(4 * n), o_aboard = take(8 * n), o_packed = take(sizeof(Packed) * n);
     const size_t o_len = take(4 * n), o_moves = take(SV_MAXLEN * n), o_nodes = take(8 * SV_MAXIT * n),
                  o_iters = take(4 * n), o_status = take(4 * n);
-    const size_t o_ovf = take((size_t)total_warps * ovf_cap * WarpStack<SV_W>::ENTRY_BYTES);
+    const size_t o_ovf = take((size_t)chain_warps * ovf_cap * WarpStack<SV_W>::ENTRY_BYTES);
     const size_t o_carry = take(4 * n), o_fbase = take(4 * n), o_fcount = take(4 * n);
     if (cudaMalloc(&sv->mem, off) != cudaSuccess) {
         delete sv;
@@ -369,7 +382,9 @@ bpida_server *bpida_server_create(const bpida_config *cfg, size_t frontier_bytes
     }
     const int exit_pct = (cfg && cfg->exit_fraction_pct > 0) ? cfg->exit_fraction_pct : 10;
     d.tune.min_rounds = (cfg && cfg->min_rounds > 0) ? cfg->min_rounds : 64;
-    d.tune.exit_threshold = std::max(1, total_warps * exit_pct / 100);
+    sv->exit_threshold = std::max(1, total_warps * exit_pct / 100);
+    sv->chain_exit_threshold = std::max(1, chain_warps * exit_pct / 100);
+    d.tune.chain_nodes = CHAIN_MIN_NODES;
     d.tune.nodes_per_record = 4096;
     d.tune.target_cap = tcap;
     d.tune.target_path = std::min(tcap, 4096);

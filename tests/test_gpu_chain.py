@@ -1,8 +1,10 @@
 """The 15-puzzle search of larger calls (one child per lane and round) at the
 edges of its dispatch and of its stacks, against the stored oracle results.
 Every output is a whole number: exact."""
+import numpy as np
 import pytest
 
+import oracle
 from paper_1705_02843_gb300 import bpida
 from paper_1705_02843_gb300 import inputs as I
 from tests.test_gpu_parity import _golden, gpu_solve
@@ -63,3 +65,34 @@ def test_very_hard_batch_stays_within_the_queues():
     for g, h in zip(got, halves):
         assert g["status"] == h["status"] == bpida.OK
         assert (g["length"], g["nodes"], g["moves"], g["solutions"]) == (h["length"], h["nodes"], h["moves"], h["solutions"])
+
+
+@pytest.mark.parametrize("driver", [0, 1])
+@pytest.mark.parametrize("n", [64, 256, 700])
+def test_easy_batches_keep_the_short_steps_kernel(n, driver):
+    """Calls of many easy boards: no step is large enough for the kernel of
+    large steps, which would be the slower one."""
+    insts = [I.make_walk(4, 9000 + i, 40) for i in range(n)]
+    tiles = [x.tiles for x in insts]
+    rc, got = gpu_solve(4, tiles, driver=driver)
+    assert rc == bpida.OK and bpida.chain_passes() == 0
+    ref = oracle.solve_batch(4, np.array(tiles[::n // 16], dtype=np.uint8), count_all=True)
+    for g, r in zip(got[::n // 16], ref):
+        assert (g["status"], g["length"], g["nodes"], g["moves"]) == (0, r.length, r.nodes, r.moves)
+
+
+@pytest.mark.parametrize("driver", [0, 1])
+def test_hard_batches_use_both_kernels(driver):
+    """Small first steps on one kernel, large ones on the other; no call of
+    fewer than 64 boards uses the latter."""
+    gold = sorted(_golden("perms15_100")["instances"], key=lambda r: sum(r["nodes"]))[:64]
+    perms = I.perms15_100()
+    for n in (63, 64):
+        rc, got = gpu_solve(4, [perms[r["index"]].tiles for r in gold[:n]], driver=driver)
+        assert rc == bpida.OK
+        if n < 64:
+            assert bpida.chain_passes() == 0
+        else:
+            assert 0 < bpida.chain_passes() < bpida.last_stats()["passes"]
+        for r, g in zip(gold, got):
+            assert (g["status"], g["length"], g["nodes"], g["solutions"]) == (0, r["length"], r["nodes"], r["solutions"])
