@@ -310,9 +310,9 @@ struct ChainGeometry {
 
 // 15-puzzle calls of at least CHAIN_MIN_N boards search their large steps
 // (CHAIN_MIN_NODES, bpida_chain.cuh) with k_search_chain, in a pass loop of
-// its own. Smaller calls are without that loop: skipping it takes about 1 % of
-// a call of easy boards (64 40-move walks 1471 us; 63 of them, without it,
-// 1449).
+// its own. Smaller calls are without that loop: passing it by takes about 1 %
+// of a call of easy boards (64 40-move walks 1462 us; 63 of them, without it,
+// 1447).
 constexpr int CHAIN_MIN_N = 64;
 // Its stack entries per lane: 20 where they fit (five 4-warp blocks per SM;
 // every block size that a caller can ask for leaves room for 13).
@@ -429,28 +429,31 @@ cudaError_t build_graph(Plan &pl, Dev<W> d, const Geometry &g, const Dev<W> &d_c
             return e;
         d.h_chain = hc;
     }
-    cudaGraphNode_t n_split, n_pass, n_adv;
+    cudaGraphNode_t n_split, n_pass[2], n_adv;
+    int loops = 1;
     *where = "split/pass/advance nodes";
     if ((e = add_kernel(&n_split, B, nullptr, 0, split_kernel<W, PDB>(g.n_cap), g_prob, dim3(split_threads(g.n_cap)), 0, d)) != cudaSuccess)
         return e;
     cudaGraph_t P;
-    if ((e = add_while(&n_pass, B, &n_split, 1, hp, &P)) != cudaSuccess)
+    if ((e = add_while(&n_pass[0], B, &n_split, 1, hp, &P)) != cudaSuccess)
         return e;
     if constexpr (W == 4 && !PDB)
         if (gc.cap) {
             cudaGraph_t PC;
-            cudaGraphNode_t n_chain, n_loop = n_pass;
+            cudaGraphNode_t n_chain;
             Dev<W> dc = d_chain;
             dc.graph = 1;
             dc.h_step = hs;
             dc.h_pass = d.h_chain;
-            if ((e = add_while(&n_pass, B, &n_loop, 1, d.h_chain, &PC)) != cudaSuccess)
+            // beside the other loop, not behind it: 8 to 16 us of a call less
+            // (64 10-to-20-move walks 418 -> 411 us)
+            if ((e = add_while(&n_pass[loops++], B, &n_split, 1, d.h_chain, &PC)) != cudaSuccess)
                 return e;
             if ((e = add_kernel(&n_chain, PC, nullptr, 0, chain_kernel(g.threads / 32), dim3(gc.grid), dim3(g.threads), gc.smem,
                                 dc)) != cudaSuccess)
                 return e;
         }
-    if ((e = add_kernel(&n_adv, B, &n_pass, 1, k_advance<W>, g_inst, b128, 0, d)) != cudaSuccess)
+    if ((e = add_kernel(&n_adv, B, n_pass, loops, k_advance<W>, g_inst, b128, 0, d)) != cudaSuccess)
         return e;
 
     cudaGraphNode_t n_search;
