@@ -88,7 +88,7 @@ struct Plan {
 };
 
 struct Workspace {
-    DevBuf state, act0, act1, ctr, scratch, count, offset, q0, q1, ctrl, desc, ovf, fuse;
+    DevBuf state, act0, act1, ctr, scratch, count, offset, queues, ctrl, desc, ovf, fuse;
     Ctrl *h_ctrl = nullptr;  // pinned copy of the control block, written at the end of each call
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
     cudaEvent_t done = nullptr;         // recorded after the last call's work
@@ -156,7 +156,7 @@ struct Workspace {
         for (auto &kv : plans)
             kv.second.destroy();
         plans.clear();
-        DevBuf *all[] = {&state, &act0, &act1, &ctr, &scratch, &count, &offset, &q0, &q1, &ctrl, &desc, &ovf,
+        DevBuf *all[] = {&state, &act0, &act1, &ctr, &scratch, &count, &offset, &queues, &ctrl, &desc, &ovf,
                          &fuse};
         for (DevBuf *b : all) {
             if (b->p)
@@ -522,9 +522,8 @@ bpida_status run(const Settings &cfg, const uint64_t *boards, int n, int *out_le
     // per-warp overflow stacks, and the hand-back queue: every warp's shared
     // and overflow stacks plus its unfinished chunk, twice over; overflowing
     // it is detected and reported as BPIDA_ENOMEM
-    const int ovf_cap = (W == 5) ? 4 * S : gc.cap ? CHAIN_OVERFLOW : 0;
-    g.Q = std::max({(size_t)n * g.C, (size_t)g.total_warps * (S + (gc.cap ? 0 : ovf_cap) + 32) * 2,
-                    (size_t)gc.total_warps * (32 * gc.cap + 32 + ovf_cap + 32) * 2, (size_t)1 << 24}) + 1024;
+    const int ovf_cap = (W == 5) ? 4 * S : 0;
+    g.Q = std::max({(size_t)n * g.C, (size_t)g.total_warps * (S + ovf_cap + 32) * 2, (size_t)1 << 24}) + 1024;
     if (g.Q > (size_t)INT_MAX / 2 || (size_t)n * 2 * g.C > (size_t)UINT32_MAX)
         return BPIDA_ENOMEM;
 
@@ -535,11 +534,10 @@ bpida_status run(const Settings &cfg, const uint64_t *boards, int n, int *out_le
     CK(ws.ensure(ws.scratch, sizeof(Rec<W>) * (size_t)n * 2 * g.C));
     CK(ws.ensure(ws.count, sizeof(int) * n));
     CK(ws.ensure(ws.offset, sizeof(int) * n));
-    CK(ws.ensure(ws.q0, sizeof(Rec<W>) * g.Q));
-    CK(ws.ensure(ws.q1, sizeof(Rec<W>) * g.Q));
+    CK(ws.ensure(ws.queues, 2 * sizeof(Rec<W>) * g.Q));
     CK(ws.ensure(ws.ctrl, sizeof(Ctrl)));
     CK(ws.ensure(ws.desc, sizeof(CallDesc)));
-    CK(ws.ensure(ws.ovf, (size_t)(gc.cap ? gc.total_warps : g.total_warps) * ovf_cap * WarpStack<W>::ENTRY_BYTES));
+    CK(ws.ensure(ws.ovf, (size_t)g.total_warps * ovf_cap * WarpStack<W>::ENTRY_BYTES));
     if (fuse)
         CK(ws.ensure(ws.fuse, (size_t)n * (sizeof(int) + FUSE_K * (2 * sizeof(unsigned long long) + sizeof(unsigned)))));
     if (!ws.h_ctrl)
@@ -558,14 +556,16 @@ bpida_status run(const Settings &cfg, const uint64_t *boards, int n, int *out_le
     d.act0 = (unsigned *)ws.act0.p;
     d.act1 = (unsigned *)ws.act1.p;
     d.scratch = (Rec<W> *)ws.scratch.p;
-    d.q0 = (Rec<W> *)ws.q0.p;
-    d.q1 = (Rec<W> *)ws.q1.p;
+    if (gc.cap)
+        g.Q -= CHAIN_OVERFLOW_RECS;  // k_search_chain's overflow stacks, behind the queues
+    d.q0 = (Rec<W> *)ws.queues.p;
+    d.q1 = d.q0 + g.Q;
     d.count = (int *)ws.count.p;
     d.offset = (int *)ws.offset.p;
     d.C = g.C;
     d.Q = (int)g.Q;
-    d.ovf = (unsigned char *)ws.ovf.p;
-    d.ovf_cap = ovf_cap;
+    d.ovf = gc.cap ? (unsigned char *)(d.q1 + g.Q) : (unsigned char *)ws.ovf.p;
+    d.ovf_cap = gc.cap ? CHAIN_OVERFLOW / gc.total_warps : ovf_cap;
     d.chain_cap = gc.cap;
     if (fuse) {
         char *p = (char *)ws.fuse.p;

@@ -169,10 +169,15 @@ struct ChainStack {
         put_if(1u, to, x, y, z, w);
     }
 };
-// Entries of a warp's overflow stack in global memory: about the open nodes of 32
-// paths of the deepest searches. With 512 the hand-back queue overflowed on a
-// batch with a board of more than 1e11 nodes.
-static constexpr int CHAIN_OVERFLOW = 4096;
+// Entries of all warps' overflow stacks in global memory, which take the room of
+// CHAIN_OVERFLOW_RECS records of each of the two hand-back queues (so that a
+// workspace is no larger than one without them). At five 4-warp blocks on 152
+// SMs a warp has 4139 entries, and the largest hand-back of a batch with a board
+// of more than 1e11 nodes is 4.7 million records, of queues that hold 12.6
+// million at least (6.1 million with 3072 entries, 8.5 with 2048, 15.0 with
+// 1024, 23.5 with 512; the time is the same from 1024 up).
+static constexpr int CHAIN_OVERFLOW_RECS = 1 << 22, CHAIN_OVERFLOW = 3 << 22;
+static_assert(sizeof(uint4) * CHAIN_OVERFLOW == 2 * sizeof(Rec<4>) * CHAIN_OVERFLOW_RECS, "overflow stacks take records' room");
 
 // A step searches with this kernel when it is predicted to expand at least
 // CHAIN_MIN_NODES nodes (k_advance's sum over the step's instances, eight

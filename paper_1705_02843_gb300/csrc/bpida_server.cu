@@ -316,9 +316,11 @@ bpida_server *bpida_server_create(const bpida_config *cfg, size_t frontier_bytes
         return nullptr;
     }
     const int total_warps = sv->grid * SV_WPB, chain_warps = sv->chain_grid * SV_WPB;
-    const int ovf_cap = CHAIN_OVERFLOW;
-    const size_t Q = std::max({(size_t)slots * C, (size_t)total_warps * (SV_S + 32) * 2,
-                               (size_t)chain_warps * (32 * SV_CAP + 32 + ovf_cap + 32) * 2, (size_t)1 << 24}) + 1024;
+    // the hand-back queues, with k_search_chain's overflow stacks in their
+    // room. (A frontier has fewer than 3 * tcap records besides goals: the
+    // queues hold every slot's.)
+    const size_t Q = std::max({(size_t)slots * C, (size_t)total_warps * (SV_S + 32) * 2, (size_t)1 << 24}) + 1024 -
+                     CHAIN_OVERFLOW_RECS;
 
     // one allocation carved into the workspace
     const size_t n = (size_t)slots;
@@ -336,7 +338,7 @@ bpida_server *bpida_server_create(const bpida_config *cfg, size_t frontier_bytes
     const size_t o_done = take(4 * n), o_aslot = take(4 * n), o_aboard = take(8 * n), o_packed = take(sizeof(Packed) * n);
     const size_t o_len = take(4 * n), o_moves = take(SV_MAXLEN * n), o_nodes = take(8 * SV_MAXIT * n),
                  o_iters = take(4 * n), o_status = take(4 * n);
-    const size_t o_ovf = take((size_t)chain_warps * ovf_cap * WarpStack<SV_W>::ENTRY_BYTES);
+    const size_t o_ovf = take(sizeof(uint4) * (size_t)CHAIN_OVERFLOW);
     const size_t o_carry = take(4 * n), o_fbase = take(4 * n), o_fcount = take(4 * n);
     if (cudaMalloc(&sv->mem, off) != cudaSuccess) {
         delete sv;
@@ -358,7 +360,7 @@ bpida_server *bpida_server_create(const bpida_config *cfg, size_t frontier_bytes
     d.C = C;
     d.Q = (int)Q;
     d.ovf = (unsigned char *)(b + o_ovf);
-    d.ovf_cap = ovf_cap;
+    d.ovf_cap = CHAIN_OVERFLOW / chain_warps;
     d.chain_cap = SV_CAP;
     d.slice = 1;
     d.carry = (unsigned *)(b + o_carry);

@@ -3,6 +3,7 @@ edges of its dispatch and of its stacks, against the stored oracle results.
 Every output is a whole number: exact."""
 import numpy as np
 import pytest
+import torch
 
 import oracle
 from paper_1705_02843_gb300 import bpida
@@ -96,3 +97,41 @@ def test_hard_batches_use_both_kernels(driver):
             assert 0 < bpida.chain_passes() < bpida.last_stats()["passes"]
         for r, g in zip(gold, got):
             assert (g["status"], g["length"], g["nodes"], g["solutions"]) == (0, r["length"], r["nodes"], r["solutions"])
+
+
+def _used(make):
+    """Device bytes that make() leaves allocated."""
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    kept = make()
+    torch.cuda.synchronize()
+    after = torch.cuda.mem_get_info()[0]
+    return before - after, kept
+
+
+QUEUES = 2 * 24 * ((1 << 24) + 1024)  # the two hand-back queues' bytes (24-byte records)
+
+
+@pytest.mark.parametrize("cfg", [dict(), dict(warps_per_block=32, stack_entries=256)])
+def test_workspace_is_no_larger_than_a_smaller_calls(cfg):
+    """The large steps' overflow stacks take room of the hand-back queues. In
+    a call's bytes: the queues, the frontiers (2 * 16388 records a board) and
+    less than 16 MiB of the rest (per-board state, the graph)."""
+    boards = torch.from_numpy(I.packed_array([I.make_walk(4, 100 + i, 30) for i in range(64)]).view(np.int64)).cuda()
+    c = bpida.make_config(4, **cfg)
+    for n in (63, 64):  # loads the kernels
+        bpida.solve(boards[:n], 4, c).synchronize()
+    for n in (63, 64):
+        bpida.release_workspace()
+        used, _ = _used(lambda: bpida.solve(boards[:n], 4, c).synchronize())
+        assert used < QUEUES + n * 2 * 16388 * 24 + (16 << 20), n
+    bpida.release_workspace()
+
+
+def test_server_memory():
+    """A server's bytes: its frontier memory, the queues, less than 16 MiB of
+    the rest (16 slots)."""
+    bpida.Server(frontier_bytes=64 << 20, max_slots=16).close()  # loads the kernels
+    used, sv = _used(lambda: bpida.Server(frontier_bytes=64 << 20, max_slots=16))
+    sv.close()
+    assert used < QUEUES + (64 << 20) + (16 << 20)
