@@ -357,6 +357,19 @@ int bpida_get_launch_log(double *ms, uint64_t *nodes, int cap);
  * (8e6). Process-wide; takes effect at the next call. */
 void bpida_set_fuse_nodes(uint64_t nodes);
 
+/* Limits of the solve calls that this host thread makes from now on
+ * (bpida_solve, bpida_solve_ex and bpida_solve_pdb, variants 0, 1 and 6), for
+ * tests of what happens at them; 0 restores a default, and a value above the
+ * default changes nothing for the first two:
+ *   queue_records    capacity of each hand-back queue: a call that overflows
+ *                    it ends with BPIDA_ENOMEM for the boards not finished
+ *   overflow_entries stack entries per warp in device memory: a warp whose
+ *                    stacks are full hands entries to the next pass
+ *   large_step_nodes predicted nodes from which a step is large (see
+ *                    bpida_get_chain_passes)
+ * Results of boards that end with BPIDA_OK do not depend on them. */
+void bpida_set_search_limits(uint64_t queue_records, uint64_t overflow_entries, uint64_t large_step_nodes);
+
 /* Free the calling device's workspaces (after waiting for their last calls)
  * and forget bpida_solve_noalloc's array address on it. */
 void bpida_release_workspace(void);

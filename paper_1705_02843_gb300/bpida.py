@@ -22,7 +22,7 @@ BLOCK_PARALLEL, PAPER_KERNEL, PSIMPLE, PSTATICLB, PFULLLB, BPSTATIC, BLOCK_MODE 
 
 EXPORTS = (
     "bpida_max_len", "bpida_max_iters", "bpida_solve", "bpida_solve_ex", "bpida_set_timing",
-    "bpida_set_fuse_nodes",
+    "bpida_set_fuse_nodes", "bpida_set_search_limits",
     "bpida_get_stats", "bpida_get_chain_passes", "bpida_get_launch_log", "bpida_release_workspace", "bpida_status_str", "bpida_solve_noalloc",
     "bpida_server_create", "bpida_server_submit", "bpida_server_poll", "bpida_server_in_flight",
     "bpida_server_get_stats", "bpida_server_clock", "bpida_server_set_time_slice", "bpida_server_destroy",
@@ -140,6 +140,8 @@ def load():
         lib.bpida_set_timing.restype = None
         lib.bpida_set_fuse_nodes.argtypes = [ctypes.c_uint64]
         lib.bpida_set_fuse_nodes.restype = None
+        lib.bpida_set_search_limits.argtypes = [ctypes.c_uint64] * 3
+        lib.bpida_set_search_limits.restype = None
         lib.bpida_get_stats.argtypes = [ctypes.POINTER(Stats)]
         lib.bpida_get_stats.restype = None
         lib.bpida_get_chain_passes.argtypes = []
@@ -205,6 +207,11 @@ def set_timing(on: bool) -> None:
 def set_fuse_nodes(nodes: int) -> None:
     """Node cap of a fused step's top threshold (0: the defaults); see bpida.h."""
     load().bpida_set_fuse_nodes(int(nodes))
+
+
+def set_search_limits(queue_records: int = 0, overflow_entries: int = 0, large_step_nodes: int = 0) -> None:
+    """Limits of this thread's later solve calls (0: the defaults); see bpida.h."""
+    load().bpida_set_search_limits(int(queue_records), int(overflow_entries), int(large_step_nodes))
 
 
 def last_stats() -> dict:

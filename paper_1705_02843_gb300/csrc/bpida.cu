@@ -58,6 +58,11 @@ struct LaunchRec {
 };
 thread_local std::vector<LaunchRec> g_launch_log;
 thread_local uint64_t g_chain_passes = 0;  // of this thread's last host-driven call
+// bpida_set_search_limits (0: the defaults)
+struct Limits {
+    uint64_t queue_records, overflow_entries, large_step_nodes;
+};
+thread_local Limits g_limits = {0, 0, 0};
 std::atomic<unsigned long long> g_fuse_nodes{0};  // 0: the defaults below
 std::mutex g_mu;
 
@@ -67,8 +72,10 @@ struct DevBuf {
 };
 
 // W, S, warps per block, n, frontier cap, hand-back percentage, min rounds, min pass time, variant,
-// fused iterations, pattern databases (their id; 0 = Manhattan distance), fused-step node cap
-typedef std::tuple<int, int, int, int, int, int, int, int, int, int, unsigned long long, unsigned long long>
+// fused iterations, pattern databases (their id; 0 = Manhattan distance), fused-step node cap, queue capacity,
+// overflow stack entries, node limit of large steps
+typedef std::tuple<int, int, int, int, int, int, int, int, int, int, unsigned long long, unsigned long long, int, int,
+                   unsigned long long>
     PlanKey;
 
 struct Plan {
@@ -564,8 +571,12 @@ bpida_status run(const Settings &cfg, const uint64_t *boards, int n, int *out_le
     d.offset = (int *)ws.offset.p;
     d.C = g.C;
     d.Q = (int)g.Q;
+    if (g_limits.queue_records && g_limits.queue_records < g.Q)
+        d.Q = (int)g_limits.queue_records;
     d.ovf = gc.cap ? (unsigned char *)(d.q1 + g.Q) : (unsigned char *)ws.ovf.p;
     d.ovf_cap = gc.cap ? CHAIN_OVERFLOW / gc.total_warps : ovf_cap;
+    if (g_limits.overflow_entries && g_limits.overflow_entries < (uint64_t)d.ovf_cap)
+        d.ovf_cap = (int)g_limits.overflow_entries;
     d.chain_cap = gc.cap;
     if (fuse) {
         char *p = (char *)ws.fuse.p;
@@ -602,7 +613,7 @@ bpida_status run(const Settings &cfg, const uint64_t *boards, int n, int *out_le
     d.tune.target_path = std::min(g.tcap, 4096);
     d.tune.growth = 8;
     d.tune.min_pass_ns = cfg.min_pass_ns;
-    d.tune.chain_nodes = gc.cap ? CHAIN_MIN_NODES : 0ull;
+    d.tune.chain_nodes = !gc.cap ? 0ull : g_limits.large_step_nodes ? g_limits.large_step_nodes : CHAIN_MIN_NODES;
     d.lut = make_move_lut<W>();
     if constexpr (PDB) {
         d.pdb.tab = cfg.pdb->tab;
@@ -638,7 +649,8 @@ bpida_status run(const Settings &cfg, const uint64_t *boards, int n, int *out_le
     const dim3 g_inst((n + 127) / 128);
     if (cfg.driver == 0) {
         const PlanKey key(W, S, cfg.wpb, n, g.tcap, cfg.exit_pct, cfg.min_rounds, cfg.min_pass_ns, cfg.variant,
-                          fuse ? 1 : 0, PDB ? cfg.pdb->id : 0ull, fuse ? d.fuse.max_nodes : 0ull);
+                          fuse ? 1 : 0, PDB ? cfg.pdb->id : 0ull, fuse ? d.fuse.max_nodes : 0ull, d.Q, d.ovf_cap,
+                          d.tune.chain_nodes);
         auto found = ws.plans.find(key);
         if (found == ws.plans.end() || !found->second.exec || found->second.gen != ws.gen) {
             ws.trim_plans();
@@ -955,6 +967,11 @@ uint64_t bpida_get_chain_passes(void)
         return g_chain_passes;
     std::lock_guard<std::mutex> lock(g_mu);
     return g_last.ws->last_call == g_last.call && g_last.ws->h_ctrl ? g_last.ws->h_ctrl->chain_passes : 0;
+}
+
+void bpida_set_search_limits(uint64_t queue_records, uint64_t overflow_entries, uint64_t large_step_nodes)
+{
+    g_limits = {queue_records, overflow_entries, large_step_nodes};
 }
 
 void bpida_set_fuse_nodes(uint64_t nodes) { g_fuse_nodes.store(nodes); }

@@ -135,3 +135,106 @@ def test_server_memory():
     used, sv = _used(lambda: bpida.Server(frontier_bytes=64 << 20, max_slots=16))
     sv.close()
     assert used < QUEUES + (64 << 20) + (16 << 20)
+
+
+@pytest.fixture
+def limits():
+    yield bpida.set_search_limits
+    bpida.set_search_limits()
+
+
+def _easiest_perms(n):
+    gold = sorted(_golden("perms15_100")["instances"], key=lambda r: sum(r["nodes"]))[:n]
+    perms = I.perms15_100()
+    return gold, [perms[r["index"]].tiles for r in gold]
+
+
+def _exact(r, g):
+    assert (g["status"], g["length"], g["nodes"], g["solutions"]) == (0, r["length"], r["nodes"], r["solutions"])
+    assert "".join(map(str, g["moves"])) == r["moves"]
+
+
+# the edges of test_block_sizes_and_stacks, with every step after the first on
+# the large steps' kernel
+@pytest.mark.parametrize("cfg", [
+    dict(), dict(warps_per_block=1), dict(warps_per_block=16), dict(warps_per_block=17),
+    dict(warps_per_block=32, stack_entries=256), dict(exit_fraction_pct=1, min_rounds=1, min_pass_us=-1),
+    dict(warps_per_block=32, stack_entries=256, split_target=1, driver=1),
+])
+def test_small_steps_on_the_large_steps_kernel(cfg, limits):
+    gold, tiles = _easiest_perms(64)
+    gpu_solve(4, tiles, **cfg)
+    large = bpida.chain_passes()
+    limits(large_step_nodes=1)
+    rc, got = gpu_solve(4, tiles, **cfg)
+    assert rc == bpida.OK and bpida.chain_passes() > large
+    for r, g in zip(gold, got):
+        _exact(r, g)
+
+
+@pytest.mark.parametrize("driver", [0, 1])
+def test_easy_boards_on_the_large_steps_kernel(driver, limits):
+    """Goals at the root and above the split depth, first solutions, budgets."""
+    tiles = [I.make_walk(4, 7000 + i, i % 44).tiles for i in range(200)]
+    ref = oracle.solve_batch(4, np.array(tiles, dtype=np.uint8), count_all=True)
+    limits(large_step_nodes=1)
+    rc, got = gpu_solve(4, tiles, driver=driver)
+    assert rc == bpida.OK and bpida.chain_passes() > 0
+    for g, r in zip(got, ref):
+        assert (g["status"], g["length"], g["nodes"], g["moves"]) == (0, r.length, r.nodes, r.moves)
+    rc, got = gpu_solve(4, tiles, driver=driver, count_all=False)
+    for g, r in zip(got, ref):
+        assert (g["status"], g["length"], g["nodes"][:-1]) == (0, r.length, r.nodes[:-1])
+        assert 1 <= g["nodes"][-1] <= r.nodes[-1]
+    budget = sorted(sum(r.nodes) for r in ref)[120]
+    rc, got = gpu_solve(4, tiles, driver=driver, node_budget=budget)
+    for g, r in zip(got, ref):
+        if sum(r.nodes) <= budget:
+            assert (g["status"], g["nodes"], g["moves"]) == (0, r.nodes, r.moves)
+        else:
+            assert g["status"] == bpida.EBUDGET and g["nodes"] == r.nodes[:len(g["nodes"])]
+
+
+@pytest.mark.parametrize("cfg", [dict(stack_entries=1024), dict(warps_per_block=32, stack_entries=384)])
+def test_full_overflow_stacks_hand_entries_to_the_next_pass(cfg, limits):
+    """Without room in the overflow stacks, full lanes hand entries back in
+    the middle of a run, and every result is the same. (With the hand-back
+    threshold at all warps, which a busy warp never sees, nothing else is
+    handed back.)"""
+    gold, tiles = _easiest_perms(64)
+    limits(large_step_nodes=1)
+    gpu_solve(4, tiles, exit_fraction_pct=100, **cfg)
+    assert bpida.last_stats()["handed_back"] == 0
+    limits(overflow_entries=1, large_step_nodes=1)
+    rc, got = gpu_solve(4, tiles, exit_fraction_pct=100, **cfg)
+    assert rc == bpida.OK and bpida.last_stats()["handed_back"] > 0
+    for r, g in zip(gold, got):
+        _exact(r, g)
+
+
+@pytest.mark.parametrize("driver", [0, 1])
+@pytest.mark.parametrize("n", [60, 64])
+def test_a_full_queue_ends_the_unfinished_boards(n, driver, limits):
+    """Both kernels on a queue of 20000 records: the boards that were not
+    finished when it overflowed end with BPIDA_ENOMEM, the others (here
+    boards of at most three moves) have their results, and the next
+    call is unharmed."""
+    gold, tiles = _easiest_perms(n - 4)
+    easy = [I.make_walk(4, 40 + i, i).tiles for i in range(4)]
+    ref = oracle.solve_batch(4, np.array(easy, dtype=np.uint8), count_all=True)
+    limits(queue_records=20000, overflow_entries=1, large_step_nodes=1)
+    rc, got = gpu_solve(4, easy + tiles, stack_entries=256, driver=driver)
+    assert rc == (bpida.ENOMEM if driver else bpida.OK)
+    assert {g["status"] for g in got} == {bpida.OK, bpida.ENOMEM}
+    for g, r in zip(got[:4], ref):
+        assert (g["status"], g["length"], g["nodes"], g["moves"]) == (0, r.length, r.nodes, r.moves)
+    for g, r in zip(got[4:], gold):
+        if g["status"] == bpida.OK:
+            _exact(r, g)
+        else:
+            assert g["length"] == -1 and g["nodes"] == r["nodes"][:len(g["nodes"])]
+    limits()
+    rc, got = gpu_solve(4, easy + tiles, driver=driver)
+    assert rc == bpida.OK
+    for g, r in zip(got[4:], gold):
+        _exact(r, g)
