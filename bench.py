@@ -69,21 +69,22 @@ WORKLOAD_DESC = {
 # 2 cycles, so above one half the ALU pipe, not issue, bounds the kernel at
 # issue peak / (2 x share)), and DRAM bytes (read + write) of the captured
 # launch, for the kernel each form runs.
-#   batched: k_search_chain, a launch of 3.0e8 nodes of a batched solve of 12
-#   random permutations: 798.3 M warp instructions; ALU share (issue 70.6 %,
-#   ALU pipe 73.5 % busy) from the same capture
-#   (profiles/k_search_chain_15puzzle_perms_batched.txt). DRAM bytes from a
-#   full capture of the four-move kernel on the 4096-board mix
-#   (profiles/k_search_15puzzle_mixed15_4096_batched.txt): frontier records,
-#   queue and counters, the same in both;
+#   batched: k_search_chain, a launch of 2.24e9 nodes of a batched solve of the
+#   4096-board mix (one of the hand-back passes of a large step): 5.670 G warp
+#   instructions, ALU pipe 74.5 % of its peak at 71.4 % issue, DRAM bytes of the
+#   same capture (profiles/k_search_chain_15puzzle_mixed15_4096_batched.txt).
+#   Passes with fewer nodes issue more per node (2.65 at 1.1e9, 2.78 at 5.3e8;
+#   the short steps' kernel 4.29), so issue utilisation computed with this
+#   figure is a lower bound;
 #   plain: the fused-iteration variant k_search<4,384,1>, the final iteration
 #   of board 0 of the mix as one pass
 #   (profiles/k_search_15puzzle_plain_fused_final_iteration.txt); its ALU
-#   share is the batched kernel's (the same step; a single-board launch's
-#   pipe fractions are skewed by its tail).
+#   share is that of k_search<4,384,0> in a steady-state launch of the mix
+#   (profiles/k_search_15puzzle_mixed15_4096_batched.txt: the same four-move
+#   step; a single-board launch's pipe fractions are skewed by its tail).
 KERNEL_COUNTERS = {
-    "batched": {"kernel": "k_search_chain<96>", "instr_per_expansion": 2.65, "alu_pipe_share": 0.52,
-                "traffic_per_launch": 10233088},
+    "batched": {"kernel": "k_search_chain<96>", "instr_per_expansion": 2.53, "alu_pipe_share": 0.522,
+                "traffic_per_launch": 20730624},
     "plain": {"kernel": "k_search<4,384,1>", "instr_per_expansion": 4.66, "alu_pipe_share": 0.386,
               "traffic_per_launch": None},
 }
