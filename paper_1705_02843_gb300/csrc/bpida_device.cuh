@@ -2318,6 +2318,7 @@ __global__ void __launch_bounds__(SMALLB ? SPLIT_THREADS_SMALL : SPLIT_THREADS) 
     // last block: frontier offsets (each thread a run of consecutive problems),
     // then open the first pass of the step
     const unsigned *act = ctrl->cur ? a.act1 : a.act0;
+    const bool chain = a.tune.chain_nodes && ctrl->chain;  // (read here: its latency is hidden by the scan's)
     const int per = (n_active + NT - 1) / NT;
     const int k0 = min(n_active, (int)threadIdx.x * per), k1 = min(n_active, k0 + per);
     int mine = 0, n_front;
@@ -2357,7 +2358,7 @@ __global__ void __launch_bounds__(SMALLB ? SPLIT_THREADS_SMALL : SPLIT_THREADS) 
         ctrl->records_total += (unsigned long long)n_front;
         __threadfence();
         if (a.graph)
-            cudaGraphSetConditional(ctrl->chain ? a.h_chain : a.h_pass, 1u);
+            cudaGraphSetConditional(chain ? a.h_chain : a.h_pass, 1u);
     }
 }
 
@@ -2588,9 +2589,10 @@ __global__ void k_advance(const Dev<W> a)
         // the next step's search kernel (path steps, whose subtrees are small,
         // predict nothing); open nodes carried over a time slice are
         // k_search_chain's to continue: only it reads its own records
-        c->chain = a.tune.chain_nodes != 0ull &&
-                   (*(volatile unsigned long long *)&c->pred >= a.tune.chain_nodes || c->n_carry > 0);
-        c->pred = 0;
+        if (a.tune.chain_nodes) {
+            c->chain = *(volatile unsigned long long *)&c->pred >= a.tune.chain_nodes || c->n_carry > 0;
+            c->pred = 0;
+        }
         c->step_again = (c->n_active > 0 && *(volatile int *)&c->err == 0) ? 1 : 0;
         __threadfence();
         if (a.graph)
