@@ -894,6 +894,8 @@ bpida_status bpida_solve_ex(const bpida_config *cfg_in, const uint64_t *boards, 
         const bpida_status r = tp::solve(ts, boards, n, out_len, out_moves, out_nodes_per_iter, out_num_iters,
                                          out_status, out_solutions, st, &stats);
         g_stats = stats;
+        g_last.ws = nullptr;  // the statistics are these, not those of an earlier graph-driven call
+        g_chain_passes = 0;
         return r;
     }
     return dispatch(cfg, boards, n, out_len, out_moves, out_nodes_per_iter, out_num_iters, out_status,

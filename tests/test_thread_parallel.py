@@ -266,3 +266,24 @@ def test_block_parallel_results_unchanged_after_ablation_calls():
     ref = oracle.solve_batch(4, np.array(tiles, dtype=np.uint8))
     for g, r in zip(sol.to_host(), ref):
         assert g["nodes"] == r.nodes and g["moves"] == r.moves
+
+
+def test_statistics_are_the_last_calls():
+    """Statistics of a thread-parallel call that follows a graph-driven call
+    are its own (the same as when it comes first), not the earlier call's."""
+    inst = I.make_walk(4, 31, 30)
+    one = torch.from_numpy(I.packed_array([inst]).view(np.int64)).cuda()
+    many = torch.from_numpy(I.packed_array([I.make_walk(4, 40 + i, 40) for i in range(64)]).view(np.int64)).cuda()
+    cfg = bpida.make_config(4, variant=bpida.PSIMPLE)
+    keys = ("steps", "passes", "records", "search_nodes", "handed_back", "max_handed_back")
+
+    def stats():
+        assert bpida.solve(one, 4, cfg).status == bpida.OK
+        torch.cuda.synchronize()
+        return {k: bpida.last_stats()[k] for k in keys}
+
+    bpida.solve(many, 4, bpida.make_config(4, driver=1))
+    first = stats()
+    bpida.solve(many, 4).synchronize()
+    assert bpida.last_stats()["search_nodes"] > first["search_nodes"]
+    assert stats() == first
