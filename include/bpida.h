@@ -173,7 +173,8 @@ typedef struct {
     double search_ms;       /* sum of search kernel durations from CUDA
                                events on the launching stream; only with
                                bpida_set_timing(1) and driver = 1 */
-    int grid_blocks;        /* search kernel grid */
+    int grid_blocks;        /* search kernel grid (15-puzzle calls of at least
+                               64 boards: that of the smaller steps' kernel) */
     int block_threads;      /* search kernel block */
     int sm_count;
     int launches;           /* kernels launched by the call */

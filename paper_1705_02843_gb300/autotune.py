@@ -2,7 +2,8 @@
 
 Tunes the search mode (a warp or a block per subtree group: bpida_config
 variant 0 or 6), the frontier cap (root-split size), warps per block,
-per-warp stack size, hand-back threshold and minimum rounds before
+per-warp stack size (in calls of 64 and more 15-puzzles that of the smaller
+steps: the large ones' kernel has its own), hand-back threshold and minimum rounds before
 hand-back by coordinate descent on measured throughput (instances/s) of a
 sample workload, in either form: "plain" (one solve call per board) or
 "batched" (one call for all). A candidate is accepted only if every result

@@ -27,15 +27,18 @@ static constexpr uint32_t M_OPEN = 1u << 28;
 //
 // What bounds it is issue, the integer ALU pipe first. Against k_search's step
 // (pop 32 nodes of a stack shared by the warp, build all four candidates of
-// each, slots from ballots) on a pass of 3e8 nodes: 2.65 warp instructions per
-// node instead of 4.29, ALU pipe 73 % of its peak, issue slots 70 % busy (20
-// warps per SM: the lanes' stacks fill shared memory); 100 random permutations
-// in one call 225.5 -> 172.4 ms, a mix of 1024 boards 115.2 -> 91.2 ms. Tried
-// and dropped: the same nodes on one stack per warp (pops and slots by ballot,
-// 196.4 ms); idle lanes paired with givers by rank, which always robs the
-// lowest lanes (mix 98.4 against 95.5 ms with partners one flipped bit away);
-// stacks of 16 entries and more warps (91.9 against 90.7 ms); runs of up to 128
-// records (92.2 against 91.2 ms, and coarser time slices in the service).
+// each, slots from ballots) on a pass of 2.2e9 nodes: 2.53 warp instructions
+// per node instead of 4.29, ALU pipe 74.5 % of its peak, issue slots 71 % busy
+// (20 warps per SM: the lanes' stacks fill shared memory). The 100 permutations
+// of seeds 1001 to 1100 in one call 158.5 -> 125.4 ms, the 4096-board mix of
+// seeds 100000 to 104095 576 -> 437 ms (all steps on k_search / the large ones
+// on this kernel, same build). Tried and dropped, on other boards and earlier
+// builds of the step: the same nodes on one stack per warp (pops and slots by
+// ballot, 196.4 ms against 172.4); idle lanes paired with givers by rank, which
+// always robs the lowest lanes (mix 98.4 against 95.5 ms with partners one
+// flipped bit away); stacks of 16 entries and more warps (91.9 against 90.7
+// ms); runs of up to 128 records (92.2 against 91.2 ms, and coarser time slices
+// in the service).
 //
 // A node is four words: the board in the blank's frame (field j holds the
 // tile of cell (p + j) mod 16, p the blank's cell, so that the neighbours up,

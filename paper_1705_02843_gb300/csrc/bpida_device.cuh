@@ -2079,9 +2079,9 @@ __global__ void __launch_bounds__(32) k_search_paper(const Dev<W> a)
 // ballots within the warp and one barrier for the warps' totals, and the
 // counts that only the end needs are reduced there. (Before, with an indexed
 // array of children and two block scans of three barriers per level, it was
-// 10 to 136 us of every step: half of the time of 5000 8-puzzles in one call,
-// 2065 -> 1710 us; one-board calls with 6-6-3 pattern databases 3.00 -> 2.71 ms,
-// one 24-puzzle 445 -> 420 us.)
+// 10 to 136 us of every step: 5000 8-puzzles in one call 2116 -> 1771 us, 16
+// 40-move walks 1046 -> 960 us, one 24-puzzle 359 -> 341 us, four one-board
+// calls with 6-6-3 pattern databases 4.93 -> 4.77 ms, each on one GPU in turn.)
 // SMALLB: blocks of 128 threads, for calls whose frontiers are short.
 template <int W, bool SMALLB = false> struct SplitShared {
     static constexpr int CAP = SMALLB ? 128 : (W <= 4) ? 512 : 384;  // records per shared level buffer

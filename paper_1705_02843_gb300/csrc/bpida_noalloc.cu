@@ -5,9 +5,10 @@
 // moment they want a solve: hosts whose device memory is entirely reserved
 // up front by a framework's pool allocator, and latency-critical loops that
 // cannot afford cudaMalloc's implicit device synchronisation. This entry
-// point serves them: it runs the same kernels as bpida_solve_ex, driven from
-// the host, with its whole workspace taken from one file-scope __device__
-// array of BPIDA_NOALLOC_SCRATCH_BYTES. It never calls cudaMalloc, cudaFree,
+// point serves them: it runs the same kernels as bpida_solve_ex does for few
+// boards (the array has no room for the 200 MB of overflow stacks of the large
+// steps' kernel), driven from the host, with its whole workspace taken from one
+// file-scope __device__ array of BPIDA_NOALLOC_SCRATCH_BYTES. It never calls cudaMalloc, cudaFree,
 // cudaMallocHost, a graph instantiation or an event creation. The caller
 // still passes device buffers for the boards and all outputs.
 //

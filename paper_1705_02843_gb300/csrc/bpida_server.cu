@@ -6,14 +6,17 @@
 // to a completion queue as soon as their instance finishes.
 //
 // One host thread per server drives the device loop:
-//   admit (k_admit) -> one threshold step (k_split, k_search passes,
-//   k_advance) -> harvest the instances that finished (k_pack)
+//   admit (k_admit) -> one threshold step (k_split, k_search or
+//   k_search_chain passes, k_advance) -> harvest the instances that
+//   finished (k_pack),
+// using the same kernels as bpida_solve_ex.
 // A step is time-sliced: once it has run for the slice, the search passes
 // stop and the open nodes of every unfinished iteration are carried into the
 // next step (k_carry_mark), so that requests whose iterations are short
 // advance, finish and free their slots without waiting for the longest
-// iteration of the batch, and new requests join sooner.
-// using the same kernels as bpida_solve_ex. The number of slots is bounded
+// iteration of the batch, and new requests join sooner. The open nodes of
+// either search kernel go on in k_search_chain, which alone reads its own.
+// The number of slots is bounded
 // by the frontier memory the caller grants (each slot owns 2*C frontier
 // records), so admission is by frontier memory.
 #include "bpida.h"
