@@ -613,7 +613,7 @@ bpida_status run(const Settings &cfg, const uint64_t *boards, int n, int *out_le
     d.tune.target_path = std::min(g.tcap, 4096);
     d.tune.growth = 8;
     d.tune.min_pass_ns = cfg.min_pass_ns;
-    d.tune.chain_nodes = !gc.cap ? 0ull : g_limits.large_step_nodes ? g_limits.large_step_nodes : CHAIN_MIN_NODES;
+    d.chain_nodes = !gc.cap ? 0ull : g_limits.large_step_nodes ? g_limits.large_step_nodes : CHAIN_MIN_NODES;
     d.lut = make_move_lut<W>();
     if constexpr (PDB) {
         d.pdb.tab = cfg.pdb->tab;
@@ -650,7 +650,7 @@ bpida_status run(const Settings &cfg, const uint64_t *boards, int n, int *out_le
     if (cfg.driver == 0) {
         const PlanKey key(W, S, cfg.wpb, n, g.tcap, cfg.exit_pct, cfg.min_rounds, cfg.min_pass_ns, cfg.variant,
                           fuse ? 1 : 0, PDB ? cfg.pdb->id : 0ull, fuse ? d.fuse.max_nodes : 0ull, d.Q, d.ovf_cap,
-                          d.tune.chain_nodes);
+                          d.chain_nodes);
         auto found = ws.plans.find(key);
         if (found == ws.plans.end() || !found->second.exec || found->second.gen != ws.gen) {
             ws.trim_plans();

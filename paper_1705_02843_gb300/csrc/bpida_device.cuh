@@ -353,7 +353,6 @@ struct Tune {
     int growth;          // expected node growth per iteration (x)
     int min_pass_ns;     // a pass hands work back only after running this long
     unsigned long long step_ns;  // serving: time slice of a step (0 = none)
-    unsigned long long chain_nodes;  // predicted nodes from which a step searches with k_search_chain (0: never)
 };
 
 // ---------------------------------------------------------------------
@@ -426,12 +425,11 @@ template <int W> struct Dev {
     Tune tune;
     MoveLut<W> lut;
     cudaGraphConditionalHandle h_step, h_pass;
-    cudaGraphConditionalHandle h_chain;  // the pass loop of steps that search with k_search_chain
     int graph;                  // 1 inside the CUDA graph (sets the loop conditions)
     unsigned *done_list;        // serving: instances that finished in this step (else null)
     unsigned char *ovf;         // per-warp overflow stacks in global memory (may be null)
     int ovf_cap;                // entries per warp overflow stack (0 = none)
-    int chain_cap;              // k_search_chain: stack entries per lane
+    int chain_cap;              // k_search_chain: stack entries per lane (0: the call does not use it)
     Fuse fuse;                  // fused iterations (fuse.jump null: one iteration per step)
     // Serving with time slices (slice = 1): an instance's iteration may run
     // over several steps. Frontier regions then belong to instance slots, not
@@ -442,6 +440,11 @@ template <int W> struct Dev {
     unsigned *carry;
     int *fbase, *fcount;
     PdbDev pdb;                 // pattern databases (solve calls with a PDB heuristic)
+    // Where chain_cap is set (last, so that other calls' kernels do not read
+    // another line of arguments): a step searches with k_search_chain from
+    // this many predicted nodes, in a pass loop of its own
+    unsigned long long chain_nodes;
+    cudaGraphConditionalHandle h_chain;
 };
 
 __device__ __forceinline__ unsigned long long global_ns();
@@ -2318,7 +2321,7 @@ __global__ void __launch_bounds__(SMALLB ? SPLIT_THREADS_SMALL : SPLIT_THREADS) 
     // last block: frontier offsets (each thread a run of consecutive problems),
     // then open the first pass of the step
     const unsigned *act = ctrl->cur ? a.act1 : a.act0;
-    const bool chain = a.tune.chain_nodes && ctrl->chain;  // (read here: its latency is hidden by the scan's)
+    const bool chain = a.chain_cap && ctrl->chain;  // (read here: its latency is hidden by the scan's)
     const int per = (n_active + NT - 1) / NT;
     const int k0 = min(n_active, (int)threadIdx.x * per), k1 = min(n_active, k0 + per);
     int mine = 0, n_front;
@@ -2554,7 +2557,7 @@ __global__ void k_advance(const Dev<W> a)
                     want = want < 1ull ? 1ull : want;
                     want = want > (unsigned long long)a.tune.target_cap ? (unsigned long long)a.tune.target_cap : want;
                     st.target = (uint32_t)want;
-                    if (a.tune.chain_nodes)
+                    if (a.chain_cap)
                         atomicAdd(&ctrl->pred, pred);
                 }
             }
@@ -2589,8 +2592,8 @@ __global__ void k_advance(const Dev<W> a)
         // the next step's search kernel (path steps, whose subtrees are small,
         // predict nothing); open nodes carried over a time slice are
         // k_search_chain's to continue: only it reads its own records
-        if (a.tune.chain_nodes) {
-            c->chain = *(volatile unsigned long long *)&c->pred >= a.tune.chain_nodes || c->n_carry > 0;
+        if (a.chain_cap) {
+            c->chain = *(volatile unsigned long long *)&c->pred >= a.chain_nodes || c->n_carry > 0;
             c->pred = 0;
         }
         c->step_again = (c->n_active > 0 && *(volatile int *)&c->err == 0) ? 1 : 0;

@@ -389,7 +389,7 @@ bpida_server *bpida_server_create(const bpida_config *cfg, size_t frontier_bytes
     d.tune.min_rounds = (cfg && cfg->min_rounds > 0) ? cfg->min_rounds : 64;
     sv->exit_threshold = std::max(1, total_warps * exit_pct / 100);
     sv->chain_exit_threshold = std::max(1, chain_warps * exit_pct / 100);
-    d.tune.chain_nodes = CHAIN_MIN_NODES;
+    d.chain_nodes = CHAIN_MIN_NODES;
     d.tune.nodes_per_record = 4096;
     d.tune.target_cap = tcap;
     d.tune.target_path = std::min(tcap, 4096);
