@@ -187,8 +187,8 @@ static_assert(sizeof(uint4) * CHAIN_OVERFLOW == 2 * sizeof(Rec<4>) * CHAIN_OVERF
 // times their last iterations), else with k_search: this one is the faster
 // one where the search itself is the time, and the slower one on short
 // searches, whose time is how soon a record spreads over a warp's lanes. Both
-// sides measured, k_search in every step / this kernel in every step / the
-// rule: 512 40-move walks 2443 / 2787 / 2443 us, 64 50-to-60-move walks 2559 /
+// sides measured, k_search in every step / this kernel in all but the first /
+// the rule: 512 40-move walks 2443 / 2787 / 2443 us, 64 50-to-60-move walks 2559 /
 // 2893 / 2562 us, 700 of them 12.52 / 12.02 / 11.84 ms, 300 boards with 1 %
 // permutations 13.07 / 12.54 / 12.36 ms, 100 permutations 430.9 / 327.9 /
 // 327.7 ms; the service, 1000 30-to-50-move walks at once 8.54 / 8.93 / 8.48

@@ -16,9 +16,8 @@
 // advance, finish and free their slots without waiting for the longest
 // iteration of the batch, and new requests join sooner. The open nodes of
 // either search kernel go on in k_search_chain, which alone reads its own.
-// The number of slots is bounded
-// by the frontier memory the caller grants (each slot owns 2*C frontier
-// records), so admission is by frontier memory.
+// The number of slots is bounded by the frontier memory the caller grants
+// (each slot owns 2*C frontier records), so admission is by frontier memory.
 #include "bpida.h"
 #include "bpida_chain.cuh"
 
