@@ -7,7 +7,8 @@ import torch
 import oracle
 from paper_1705_02843_gb300 import bpida
 from paper_1705_02843_gb300 import inputs as I
-from tests.test_gpu_parity import _golden, gpu_solve
+from tests.test_gpu_parity import gpu_solve
+from tests.test_gpu_parity import _golden
 
 pytestmark = pytest.mark.gpu
 
